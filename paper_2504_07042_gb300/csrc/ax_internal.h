@@ -131,7 +131,7 @@ cudaError_t setup_geometry(const Ctx &c, const double *vertices, void *geo, void
 cudaError_t setup_node_coords(const Ctx &c, const double *vertices, double *xyz, cudaStream_t s);
 // Y = w|J| F per node (GLL-lumped mass); F, Y float64 when f64 else float32.
 cudaError_t setup_mass(const Ctx &c, const double *vertices, const void *F, void *Y, bool f64, cudaStream_t s);
-// diag[e][l] = e_l^T A^(e) e_l from the factors (computed in FP64 into a temporary).
+// diag[e][l] = e_l^T A^(e) e_l in FP64 arithmetic from the vertices (one launch, no temporary).
 cudaError_t setup_diag(const Ctx &c, const double *vertices, void *diag, bool f64, cudaStream_t s);
 
 // Gather-scatter and CG (ax_gs.cu).

@@ -248,25 +248,147 @@ __global__ void mass_kernel(int64_t E, int N1, const double *__restrict__ V, con
 // Diagonal of the element matrix D^T G D at node l = (i,j,k):
 //   sum_n (D[n][i]^2 g00(n,j,k) + D[n][j]^2 g11(i,n,k) + D[n][k]^2 g22(i,j,n))
 //   + 2 (D[i][i] D[j][j] g01 + D[i][i] D[k][k] g02 + D[j][j] D[k][k] g12)(l)
-template <typename T>
-__global__ void diag_kernel(int64_t E, int N1, const double *__restrict__ G, T *__restrict__ out) {
-  const int64_t n3 = (int64_t)N1 * N1 * N1;
-  const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gidx >= E * n3) return;
-  const int64_t e = gidx / n3;
-  const int l = (int)(gidx % n3), i = l % N1, j = (l / N1) % N1, k = l / (N1 * N1);
-  const double *cD = c_D + tab_off_D(N1);
-  const double *Ge = G + e * 7 * n3;
-  double d = 0.0;
-  for (int n = 0; n < N1; ++n) {
-    const double a = cD[n * N1 + i], b = cD[n * N1 + j], c = cD[n * N1 + k];
-    d += a * a * Ge[0 * n3 + n + j * N1 + k * N1 * N1];
-    d += b * b * Ge[3 * n3 + i + n * N1 + k * N1 * N1];
-    d += c * c * Ge[5 * n3 + i + j * N1 + n * N1 * N1];
+//
+// One thread per (i,j), all its k: bound by the FP64 pipe (2 operations per
+// clock and SM), so the split keeps the FP64 operations few.  The Jacobian of
+// the trilinear map is formed from its monomial coefficients
+//   x = x0 + A r + B s + C t + D rs + E rt + F st + G rst  (Eq. 8)
+// (8 additions per coefficient, shared by the element), in the columns
+//   J0 = (A + D s) + t (E + G s),  J1 = (B + D r) + t (F + G r),
+//   J2 = C + E r + F s + G r s,
+// of which only six multiply-adds change along k; with the cofactor rows
+// c0 = J1 x J2, c1 = J2 x J0, c2 = J0 x J1, det J = J2 . c2 and
+// g_ab = (w / det J) c_a . c_b.  g00 and g11 are summed along their own
+// directions through shared memory, g22 in the thread's own registers.
+// About 60 + 3 N1 FP64 operations per node.  The form it replaces (all seven
+// factors of every node by the discrete Jacobian of Sec. 3.2, N1 map
+// evaluations per direction and node, written to and read back from HBM)
+// took 200 N1 and more, 18.8 ms for 16 meshes of orders 3 to 9 (7.9M nodes)
+// on GB300; a batched solve of 20 iterations on them, which starts with it,
+// went from 26.4 to 8.1 ms.
+template <int N1>
+struct DiagShape {
+  static constexpr int F = N1 * N1, n3 = F * N1, EPB = F >= 128 ? 1 : 128 / F, threads = F * EPB;
+  static constexpr int P = N1 + 1;                // padded row of the shared factors
+  static constexpr int ES = F * P;                // padded element
+  static constexpr size_t words = 2 * (size_t)EPB * ES + EPB * 21 + F;  // g00, g11, coefficients, D^2
+};
+template <typename T, int N1>
+__global__ void __launch_bounds__(DiagShape<N1>::threads)
+    diag_kernel(int64_t E, const double *__restrict__ V, T *__restrict__ out) {
+  using Sh = DiagShape<N1>;
+  constexpr int F = Sh::F, EPB = Sh::EPB, P = Sh::P;
+  extern __shared__ double sm_diag[];
+  double *g00 = sm_diag, *g11 = g00 + EPB * Sh::ES, *coef = g11 + EPB * Sh::ES, *D2 = coef + EPB * 21;
+  const double *cD = c_D + tab_off_D(N1), *cx = c_x + tab_off_v(N1), *cw = c_w + tab_off_v(N1);
+  const int tid = threadIdx.x, z = tid / F, q = tid % F, i = q % N1, j = q / N1;
+  for (int m = tid; m < F; m += Sh::threads) D2[m] = cD[m] * cD[m];
+  const double r = cx[i], s = cx[j], wij = cw[i] * cw[j];
+  const double di = cD[i * N1 + i], dj = cD[j * N1 + j];
+  const int64_t nblk = (E + EPB - 1) / EPB;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    const int64_t e0 = blk * EPB;
+    const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
+    // monomial coefficients: (1/8) sum_v sigma(v) (V_v - V_0), as trilinear_coeffs_kernel
+    for (int m = tid; m < nel * 21; m += Sh::threads) {
+      const int el = m / 21, mono = (m % 21) / 3, c = m % 3;
+      const int use = mono < 2 ? mono + 1 : mono == 2 ? 4 : mono == 3 ? 3 : mono + 1;  // 1 2 4 3 5 6 7
+      const double *Ve = V + 24 * (e0 + el);
+      double acc = 0.0;
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        const double d = Ve[3 * v + c] - Ve[c];
+        acc += (__popc(use & ~v) & 1) ? -d : d;
+      }
+      coef[m] = acc * 0.125;
+    }
+    __syncthreads();
+    const bool live = z < nel;
+    double y[N1];
+    if (live) {
+      const double *M = coef + z * 21;  // A B C D E F G
+      double E0[3], E1[3], F0[3], F1[3], J2[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        E0[c] = fma(M[9 + c], s, M[c]);
+        E1[c] = fma(M[18 + c], s, M[12 + c]);
+        F0[c] = fma(M[9 + c], r, M[3 + c]);
+        F1[c] = fma(M[18 + c], r, M[15 + c]);
+        J2[c] = fma(E1[c], r, fma(M[15 + c], s, M[6 + c]));
+      }
+#pragma unroll
+      for (int k = 0; k < N1; ++k) y[k] = 0.0;
+      double *g0 = g00 + z * Sh::ES + i + P * j, *g1 = g11 + z * Sh::ES + i + P * j;
+#pragma unroll
+      for (int k = 0; k < N1; ++k) {
+        const double t = cx[k], dk = cD[k * N1 + k];
+        double J0[3], J1[3], c0[3], c1[3], c2[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          J0[c] = fma(t, E1[c], E0[c]);
+          J1[c] = fma(t, F1[c], F0[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int a = (c + 1) % 3, b = (c + 2) % 3;
+          c0[c] = J1[a] * J2[b] - J1[b] * J2[a];
+          c1[c] = J2[a] * J0[b] - J2[b] * J0[a];
+          c2[c] = J0[a] * J1[b] - J0[b] * J1[a];
+        }
+        const double det = J2[0] * c2[0] + J2[1] * c2[1] + J2[2] * c2[2];
+        const double lam = wij * cw[k] / det;
+        auto dot = [](const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+        g0[P * N1 * k] = lam * dot(c0, c0);
+        g1[P * N1 * k] = lam * dot(c1, c1);
+        const double g22 = lam * dot(c2, c2);
+        // D[i][i] (D[j][j] g01 + D[k][k] g02) + D[j][j] D[k][k] g12
+        const double cross = di * (dj * dot(c0, c1) + dk * dot(c0, c2)) + dj * dk * dot(c1, c2);
+        y[k] = fma(2.0 * lam, cross, y[k]);
+#pragma unroll
+        for (int n = 0; n < N1; ++n) y[n] = fma(D2[k * N1 + n], g22, y[n]);
+      }
+    }
+    __syncthreads();  // every g00, g11 is in place
+    if (live) {
+      T *o = out + (e0 + z) * (int64_t)Sh::n3 + i + N1 * j;
+#pragma unroll 1
+      for (int n = 0; n < N1; ++n) {
+        const double a = D2[n * N1 + i], b = D2[n * N1 + j];
+        const double *g0 = g00 + z * Sh::ES + n + P * j, *g1 = g11 + z * Sh::ES + i + P * n;
+#pragma unroll
+        for (int k = 0; k < N1; ++k) y[k] = fma(a, g0[P * N1 * k], fma(b, g1[P * N1 * k], y[k]));
+      }
+#pragma unroll
+      for (int k = 0; k < N1; ++k) o[F * k] = (T)y[k];
+    }
+    __syncthreads();  // the next block reuses the shared buffers
   }
-  const double di = cD[i * N1 + i], dj = cD[j * N1 + j], dk = cD[k * N1 + k];
-  d += 2.0 * (di * dj * Ge[1 * n3 + l] + di * dk * Ge[2 * n3 + l] + dj * dk * Ge[4 * n3 + l]);
-  out[gidx] = (T)d;
+}
+
+template <typename T, int N1>
+cudaError_t launch_diag(int64_t E, const double *V, T *out, cudaStream_t s) {
+  using Sh = DiagShape<N1>;
+  constexpr size_t bytes = Sh::words * sizeof(double);
+  const int64_t nblk = (E + Sh::EPB - 1) / Sh::EPB;
+  const unsigned grid = (unsigned)(nblk < 0x7fffffffLL ? nblk : 0x7fffffffLL);
+  if (bytes > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(diag_kernel<T, N1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+  }
+  diag_kernel<T, N1><<<grid, Sh::threads, bytes, s>>>(E, V, out);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_diag_n(int N1, int64_t E, const double *V, T *out, cudaStream_t s) {
+  switch (N1) {
+#define AX_DIAG(n) \
+  case n: return launch_diag<T, n>(E, V, out, s);
+    AX_DIAG(2) AX_DIAG(3) AX_DIAG(4) AX_DIAG(5) AX_DIAG(6) AX_DIAG(7) AX_DIAG(8) AX_DIAG(9)
+    AX_DIAG(10) AX_DIAG(11) AX_DIAG(12) AX_DIAG(13) AX_DIAG(14) AX_DIAG(15) AX_DIAG(16)
+#undef AX_DIAG
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 static unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
@@ -337,25 +459,9 @@ cudaError_t setup_mass(const Ctx &c, const double *V, const void *F, void *Y, bo
 }
 
 cudaError_t setup_diag(const Ctx &c, const double *V, void *diag, bool f64, cudaStream_t s) {
-  const int64_t nodes = c.E * (int64_t)c.n3;
-  if (nodes == 0) return cudaSuccess;
-  double *G = nullptr;
-  int *flags = nullptr;
-  cudaError_t e = cudaMalloc(&G, sizeof(double) * 7 * nodes);
-  if (e == cudaSuccess) e = cudaMalloc(&flags, 4 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 4 * sizeof(int), s);
-  if (e == cudaSuccess) {
-    setup::stored_factors_kernel<<<setup::grid_for(nodes, 256), 256, 0, s>>>(c.E, c.N1, V, G, setup::kF64, flags);
-    if (f64)
-      setup::diag_kernel<double><<<setup::grid_for(nodes, 256), 256, 0, s>>>(c.E, c.N1, G, (double *)diag);
-    else
-      setup::diag_kernel<float><<<setup::grid_for(nodes, 256), 256, 0, s>>>(c.E, c.N1, G, (float *)diag);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(G);
-  cudaFree(flags);
-  return e;
+  if (c.E == 0) return cudaSuccess;
+  return f64 ? setup::launch_diag_n<double>(c.N1, c.E, V, (double *)diag, s)
+             : setup::launch_diag_n<float>(c.N1, c.E, V, (float *)diag, s);
 }
 
 }  // namespace ax
