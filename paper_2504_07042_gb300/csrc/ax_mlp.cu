@@ -13,6 +13,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -53,33 +54,64 @@ __global__ void transpose_bf16(int R, int C, const __nv_bfloat16 *__restrict__ i
   }
 }
 
-// dY = (Y - T) / (M * O) as bf16; partial sums of (Y - T)^2 per block
-__global__ void loss_grad(int M, int O, const float *__restrict__ Y, const float *__restrict__ T,
-                          __nv_bfloat16 *__restrict__ dY, float *__restrict__ part) {
-  __shared__ float sh[256];
-  float s = 0.0f;
-  const float inv = 1.0f / ((float)M * (float)O);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)M * O; i += (int64_t)gridDim.x * blockDim.x) {
-    const float d = Y[i] - T[i];
-    s += d * d;
-    dY[i] = __float2bfloat16_rn(d * inv);
+// Gradients from their partial sums, everything added in a fixed order:
+// weights g[i] = sum over the batch splits of part[s][i] (gemm_dw_kernel),
+// biases db[n] = sum over 32-row blocks of the column sums the GEMM epilogues
+// left, and the loss's sum of squares.  Blocks [0, nw): weights, one float4
+// per thread; then 32 columns of a bias per block (8 strided sums per
+// column); the last block: the loss.
+struct GradSum {
+  const float *part;             // [splits][np]
+  const float *col[3];           // per layer: [rows32][512] column sums
+  const float *sq;               // [nsq]
+  float *g;
+  double *loss_sq;
+  int64_t np, woff[3], wlen[3], boff[3];
+  int splits, rows32, nsq, nw;
+};
+__global__ void __launch_bounds__(256) grad_reduce_kernel(const __grid_constant__ GradSum a) {
+  __shared__ float sh[8][32];
+  const int tid = threadIdx.x;
+  if ((int)blockIdx.x < a.nw) {
+    int64_t i = ((int64_t)blockIdx.x * 256 + tid) * 4;  // over the three weight ranges, one after the other
+    int p = 0;
+    while (p < 3 && i >= a.wlen[p]) i -= a.wlen[p++];
+    if (p == 3) return;
+    i += a.woff[p];
+    float4 s = *reinterpret_cast<const float4 *>(a.part + i);
+    for (int q = 1; q < a.splits; ++q) {
+      const float4 v = *reinterpret_cast<const float4 *>(a.part + q * a.np + i);
+      s.x += v.x;
+      s.y += v.y;
+      s.z += v.z;
+      s.w += v.w;
+    }
+    *reinterpret_cast<float4 *>(a.g + i) = s;
+    return;
   }
-  sh[threadIdx.x] = s;
+  const int bb = (int)blockIdx.x - a.nw;
+  if (bb < 3 * (kHid / 32)) {
+    const int p = bb / (kHid / 32), n = (bb % (kHid / 32)) * 32 + (tid & 31), k = tid >> 5;
+    float s = 0.0f;
+    for (int r = k; r < a.rows32; r += 8) s += a.col[p][(size_t)r * kHid + n];
+    sh[k][tid & 31] = s;
+    __syncthreads();
+    if (k == 0) {
+      for (int q = 1; q < 8; ++q) s += sh[q][tid];
+      a.g[a.boff[p] + n] = s;
+    }
+    return;
+  }
+  __shared__ double shd[256];
+  double s = 0.0;
+  for (int q = tid; q < a.nsq; q += 256) s += (double)a.sq[q];
+  shd[tid] = s;
   __syncthreads();
   for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    if (tid < w) shd[tid] += shd[tid + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-// db[n] = sum_m dZ[m][n] (fixed order: one thread per column, rows in order)
-__global__ void colsum_bf16(int M, int N, const __nv_bfloat16 *__restrict__ dZ, float *__restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.0f;
-  for (int m = 0; m < M; ++m) s += __bfloat162float(dZ[(size_t)m * N + n]);
-  db[n] = s;
+  if (tid == 0) *a.loss_sq = shd[0];
 }
 
 // Adam on a flat FP32 parameter vector; w, m, v updated in place
@@ -445,9 +477,13 @@ struct ax_mlp {
   __nv_bfloat16 *Wb[3] = {nullptr, nullptr, nullptr}, *WTb[3] = {nullptr, nullptr, nullptr};
   // activations for a batch of up to cap rows
   int64_t cap = 0;
-  float *Z1 = nullptr, *Z2 = nullptr, *Y = nullptr, *part = nullptr;
-  __nv_bfloat16 *H1 = nullptr, *H2 = nullptr, *dY = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *T1 = nullptr,
-                *T2 = nullptr;
+  float *Y = nullptr;
+  __nv_bfloat16 *H1 = nullptr, *H2 = nullptr;
+  // backward pass, for a batch of up to gcap rows
+  int64_t gcap = 0;
+  float *Z1 = nullptr, *Z2 = nullptr, *sq = nullptr, *col = nullptr, *part = nullptr;
+  __nv_bfloat16 *dY = nullptr, *dZ1 = nullptr, *dZ2 = nullptr;
+  double *loss_sq = nullptr;
   int64_t adam_t = 0;
   int *derr = nullptr;  // device error word of the GEMM kernels (bounded waits that ran out)
   std::string err;
@@ -505,84 +541,139 @@ cudaError_t refresh_bf16(ax_mlp *m, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// hidden activations and output of the forward pass
 cudaError_t ensure_cap(ax_mlp *m, int64_t rows) {
   if (rows <= m->cap) return cudaSuccess;
-  cudaFree(m->Z1); cudaFree(m->Z2); cudaFree(m->Y); cudaFree(m->part);
-  cudaFree(m->H1); cudaFree(m->H2); cudaFree(m->dY); cudaFree(m->dZ1); cudaFree(m->dZ2); cudaFree(m->T1); cudaFree(m->T2);
+  cudaFree(m->Y); cudaFree(m->H1); cudaFree(m->H2);
+  m->Y = nullptr;
+  m->H1 = m->H2 = nullptr;
   m->cap = 0;
   const int64_t r = (rows + 127) / 128 * 128;
-  cudaError_t e = cudaMalloc(&m->Z1, sizeof(float) * r * kHid);
-  if (e == cudaSuccess) e = cudaMalloc(&m->Z2, sizeof(float) * r * kHid);
-  if (e == cudaSuccess) e = cudaMalloc(&m->Y, sizeof(float) * r * kOut);
-  if (e == cudaSuccess) e = cudaMalloc(&m->part, sizeof(float) * 1024);
+  cudaError_t e = cudaMalloc(&m->Y, sizeof(float) * r * kOut);
   if (e == cudaSuccess) e = cudaMalloc(&m->H1, sizeof(__nv_bfloat16) * r * kHid);
   if (e == cudaSuccess) e = cudaMalloc(&m->H2, sizeof(__nv_bfloat16) * r * kHid);
-  if (e == cudaSuccess) e = cudaMalloc(&m->dY, sizeof(__nv_bfloat16) * r * kOut);
-  if (e == cudaSuccess) e = cudaMalloc(&m->dZ1, sizeof(__nv_bfloat16) * r * kHid);
-  if (e == cudaSuccess) e = cudaMalloc(&m->dZ2, sizeof(__nv_bfloat16) * r * kHid);
-  // transposes: the largest is [kInPad][r]
-  if (e == cudaSuccess) e = cudaMalloc(&m->T1, sizeof(__nv_bfloat16) * r * kInPad);
-  if (e == cudaSuccess) e = cudaMalloc(&m->T2, sizeof(__nv_bfloat16) * r * kInPad);
   if (e == cudaSuccess) m->cap = r;
   return e;
 }
 
-// forward of M rows of X (bf16 [M][kInPad]) -> m->Y (f32 [M][kOut])
-// (skip: optional device flag; when nonzero the three GEMMs do nothing;
+// tiles of the three weight gradients (kDwBN columns of the layer's input each)
+int dw_tiles() {
+  int t = 0;
+  for (int l = 0; l < 3; ++l) t += (kRows[l] / tc::kBM) * ((kCols[l] + tc::kDwBN - 1) / tc::kDwBN);
+  return t;
+}
+
+// the backward pass's buffers: pre-activations, back-propagated gradients,
+// the epilogues' column sums and squares, and the weight gradients' partial
+// sums (one parameter vector per batch split, at most SMs / tiles of them)
+cudaError_t ensure_grad_cap(ax_mlp *m, int64_t rows) {
+  cudaError_t e = ensure_cap(m, rows);
+  if (e != cudaSuccess || rows <= m->gcap) return e;
+  cudaFree(m->Z1); cudaFree(m->Z2); cudaFree(m->sq); cudaFree(m->col);
+  cudaFree(m->dY); cudaFree(m->dZ1); cudaFree(m->dZ2);
+  m->Z1 = m->Z2 = m->sq = m->col = nullptr;
+  m->dY = m->dZ1 = m->dZ2 = nullptr;
+  m->gcap = 0;
+  const int64_t r = (rows + 127) / 128 * 128;
+  e = cudaMalloc(&m->Z1, sizeof(float) * r * kHid);
+  if (e == cudaSuccess) e = cudaMalloc(&m->Z2, sizeof(float) * r * kHid);
+  if (e == cudaSuccess) e = cudaMalloc(&m->dY, sizeof(__nv_bfloat16) * r * kOut);
+  if (e == cudaSuccess) e = cudaMalloc(&m->dZ1, sizeof(__nv_bfloat16) * r * kHid);
+  if (e == cudaSuccess) e = cudaMalloc(&m->dZ2, sizeof(__nv_bfloat16) * r * kHid);
+  if (e == cudaSuccess) e = cudaMalloc(&m->col, sizeof(float) * 3 * (r / 32) * kHid);
+  if (e == cudaSuccess) e = cudaMalloc(&m->sq, sizeof(float) * tc::gemm_tiles((int)r, kOut) * tc::kEpiWarps);
+  if (e == cudaSuccess && !m->part)
+    e = cudaMalloc(&m->part, sizeof(float) * m->np * std::max(1, tc::sm_count() / dw_tiles()));
+  if (e == cudaSuccess && !m->loss_sq) e = cudaMalloc(&m->loss_sq, sizeof(double));
+  if (e == cudaSuccess) m->gcap = r;
+  return e;
+}
+
+// the two hidden layers of M rows of X (bf16 [M][kInPad]) -> m->H2
+// (skip: optional device flag; when nonzero the GEMMs do nothing;
 // keep_z: store the pre-activations for a backward pass)
-cudaError_t forward(ax_mlp *m, const __nv_bfloat16 *X, int64_t M, cudaStream_t s, const double *skip = nullptr,
-                    bool keep_z = false) {
+cudaError_t hidden(ax_mlp *m, const __nv_bfloat16 *X, int64_t M, cudaStream_t s, const double *skip, bool keep_z) {
   GemmOut o1;
   o1.Cf = keep_z ? m->Z1 : nullptr; o1.Hb = m->H1; o1.bias = m->p + m->off[1]; o1.ldc = kHid; o1.skip = skip;
   cudaError_t e = tc::gemm<kEpiGelu>((int)M, kHid, kInPad, X, m->Wb[0], o1, m->derr, s);
   GemmOut o2;
   o2.Cf = keep_z ? m->Z2 : nullptr; o2.Hb = m->H2; o2.bias = m->p + m->off[3]; o2.ldc = kHid; o2.skip = skip;
   if (e == cudaSuccess) e = tc::gemm<kEpiGelu>((int)M, kHid, kHid, m->H1, m->Wb[1], o2, m->derr, s);
+  return e;
+}
+
+// forward of M rows of X -> Y (f32 [M][kOut], 16-byte aligned)
+cudaError_t forward(ax_mlp *m, const __nv_bfloat16 *X, int64_t M, float *Y, cudaStream_t s,
+                    const double *skip = nullptr) {
+  cudaError_t e = hidden(m, X, M, s, skip, false);
   GemmOut o3;
-  o3.Cf = m->Y; o3.bias = m->p + m->off[5]; o3.ldc = kOut; o3.skip = skip;
+  o3.Cf = Y; o3.bias = m->p + m->off[5]; o3.ldc = kOut; o3.skip = skip;
   if (e == cudaSuccess) e = tc::gemm<kEpiF32>((int)M, kOut, kHid, m->H2, m->Wb[2], o3, m->derr, s);
   return e;
 }
 
-// forward + backward of M rows (M a multiple of 32): gradients into m->g; loss partials in m->part
+// forward + backward of M rows: gradients into m->g, the sum of squared
+// errors into m->loss_sq.  Seven launches: three layers (the last one's
+// epilogue forms dY and the loss), two back-propagations (every epilogue
+// leaves the column sums of what it writes: the bias gradients), the three
+// weight gradients, and the sums.
 cudaError_t forward_backward(ax_mlp *m, const __nv_bfloat16 *X, const float *T, int64_t M, cudaStream_t s) {
-  cudaError_t e = forward(m, X, M, s, nullptr, true);
-  if (e != cudaSuccess) return e;
-  loss_grad<<<1024, 256, 0, s>>>((int)M, kOut, m->Y, T, m->dY, m->part);
-  const dim3 tb(32, 8);
-  auto tr = [&](int R, int C, const __nv_bfloat16 *in, __nv_bfloat16 *out) {
-    transpose_bf16<<<dim3((C + 31) / 32, (R + 31) / 32), tb, 0, s>>>(R, C, in, C, out, R);
-  };
-  float *g = m->g;
-  // layer 3: dW3 = dY^T H2, db3 = colsum dY, dZ2 = (dY W3) * gelu'(Z2)
-  tr((int)M, kOut, m->dY, m->T1);
-  tr((int)M, kHid, m->H2, m->T2);
-  GemmOut w3;
-  w3.Cf = g + m->off[4]; w3.ldc = kHid;
-  e = tc::gemm<kEpiF32>(kOut, kHid, (int)M, m->T1, m->T2, w3, m->derr, s);
-  colsum_bf16<<<gfor(kOut), 256, 0, s>>>((int)M, kOut, m->dY, g + m->off[5]);
+  cudaError_t e = hidden(m, X, M, s, nullptr, true);
+  if (e == cudaSuccess && ((uintptr_t)T & 15)) {  // the loss epilogue reads 16-byte vectors
+    e = cudaMemcpyAsync(m->Y, T, sizeof(float) * M * kOut, cudaMemcpyDeviceToDevice, s);
+    T = m->Y;
+  }
+  const int64_t rows32 = (M + 31) / 32, colp = rows32 * kHid;
+  // layer 3: dY = (Y - T) / (M O), db3; dZ2 = (dY W3) * gelu'(Z2), db2
+  GemmOut o3;
+  o3.Hb = m->dY; o3.Zin = T; o3.bias = m->p + m->off[5]; o3.ldc = kOut;
+  o3.scale = 1.0f / ((float)M * (float)kOut); o3.sq = m->sq; o3.colsum = m->col + 2 * colp;
+  if (e == cudaSuccess) e = tc::gemm<kEpiLoss>((int)M, kOut, kHid, m->H2, m->Wb[2], o3, m->derr, s);
   GemmOut d2;
-  d2.Hb = m->dZ2; d2.Zin = m->Z2; d2.ldc = kHid;
+  d2.Hb = m->dZ2; d2.Zin = m->Z2; d2.ldc = kHid; d2.colsum = m->col + colp;
   if (e == cudaSuccess) e = tc::gemm<kEpiDGelu>((int)M, kHid, kOut, m->dY, m->WTb[2], d2, m->derr, s);
-  // layer 2
-  tr((int)M, kHid, m->dZ2, m->T1);
-  tr((int)M, kHid, m->H1, m->T2);
-  GemmOut w2;
-  w2.Cf = g + m->off[2]; w2.ldc = kHid;
-  if (e == cudaSuccess) e = tc::gemm<kEpiF32>(kHid, kHid, (int)M, m->T1, m->T2, w2, m->derr, s);
-  colsum_bf16<<<gfor(kHid), 256, 0, s>>>((int)M, kHid, m->dZ2, g + m->off[3]);
   GemmOut d1;
-  d1.Hb = m->dZ1; d1.Zin = m->Z1; d1.ldc = kHid;
+  d1.Hb = m->dZ1; d1.Zin = m->Z1; d1.ldc = kHid; d1.colsum = m->col;
   if (e == cudaSuccess) e = tc::gemm<kEpiDGelu>((int)M, kHid, kHid, m->dZ2, m->WTb[1], d1, m->derr, s);
-  // layer 1
-  tr((int)M, kHid, m->dZ1, m->T1);
-  tr((int)M, kInPad, X, m->T2);
-  GemmOut w1;
-  w1.Cf = g + m->off[0]; w1.ldc = kInPad;
-  if (e == cudaSuccess) e = tc::gemm<kEpiF32>(kHid, kInPad, (int)M, m->T1, m->T2, w1, m->derr, s);
-  colsum_bf16<<<gfor(kHid), 256, 0, s>>>((int)M, kHid, m->dZ1, g + m->off[1]);
-  if (e == cudaSuccess) e = cudaGetLastError();
-  return e;
+  if (e != cudaSuccess) return e;
+  // dW1 = dZ1^T X, dW2 = dZ2^T H1, dW3 = dY^T H2
+  tc::DwArgs w;
+  const __nv_bfloat16 *dz[3] = {m->dZ1, m->dZ2, m->dY}, *h[3] = {X, m->H1, m->H2};
+  w.first[0] = 0;
+  for (int l = 0; l < 3; ++l) {
+    if (!tc::make_map_mn(&w.a[l], dz[l], (int)M, kRows[l]) || !tc::make_map_mn(&w.b[l], h[l], (int)M, kCols[l]))
+      return cudaErrorInvalidValue;
+    w.n[l] = kRows[l];
+    w.k[l] = kCols[l];
+    w.off[l] = m->off[2 * l];
+    w.first[l + 1] = w.first[l] + (kRows[l] / tc::kBM) * ((kCols[l] + tc::kDwBN - 1) / tc::kDwBN);
+  }
+  w.M = (int)M;
+  w.splits = tc::dw_splits(w.first[3], (int)M);
+  w.np = m->np;
+  w.part = m->part;
+  e = tc::gemm_dw(w, m->derr, s);
+  if (e != cudaSuccess) return e;
+  GradSum a;
+  a.part = m->part;
+  a.sq = m->sq;
+  a.g = m->g;
+  a.loss_sq = m->loss_sq;
+  a.np = m->np;
+  int64_t nw = 0;
+  for (int l = 0; l < 3; ++l) {
+    a.col[l] = m->col + l * colp;
+    a.woff[l] = m->off[2 * l];
+    a.wlen[l] = (int64_t)kRows[l] * kCols[l];
+    a.boff[l] = m->off[2 * l + 1];
+    nw += a.wlen[l];
+  }
+  a.splits = w.splits;
+  a.rows32 = (int)rows32;
+  a.nsq = tc::gemm_tiles((int)M, kOut) * tc::kEpiWarps;
+  a.nw = (int)((nw / 4 + 255) / 256);
+  grad_reduce_kernel<<<a.nw + 3 * (kHid / 32) + 1, 256, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -668,8 +759,11 @@ ax_status ax_mlp_forward(ax_mlp *m, const void *X_bf16, float *Y, int64_t M, voi
   if (!m || !X_bf16 || !Y || M < 0) return mfail(m, AX_EINVAL, "ax_mlp_forward: bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = ensure_cap(m, M);
-  if (e == cudaSuccess) e = forward(m, (const __nv_bfloat16 *)X_bf16, M, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(Y, m->Y, sizeof(float) * M * kOut, cudaMemcpyDeviceToDevice, s);
+  // the last GEMM writes the caller's Y; one that is not 16-byte aligned gets a copy
+  const bool direct = ((uintptr_t)Y & 15) == 0;
+  if (e == cudaSuccess) e = forward(m, (const __nv_bfloat16 *)X_bf16, M, direct ? Y : m->Y, s);
+  if (e == cudaSuccess && !direct)
+    e = cudaMemcpyAsync(Y, m->Y, sizeof(float) * M * kOut, cudaMemcpyDeviceToDevice, s);
   return e == cudaSuccess ? AX_OK : mcuda(m, e, "ax_mlp_forward");
 }
 
@@ -678,16 +772,14 @@ ax_status ax_mlp_grad(ax_mlp *m, const void *X_bf16, const float *T, int64_t M, 
   if (!m || !X_bf16 || !T || !loss || !grads || M < 32 || M % 32)
     return mfail(m, AX_EINVAL, "ax_mlp_grad: bad arguments (M must be a positive multiple of 32)");
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = ensure_cap(m, M);
+  cudaError_t e = ensure_grad_cap(m, M);
   if (e == cudaSuccess) e = forward_backward(m, (const __nv_bfloat16 *)X_bf16, T, M, s);
-  std::vector<float> part(1024);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(part.data(), m->part, sizeof(float) * 1024, cudaMemcpyDeviceToHost, s);
+  double sq = 0.0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&sq, m->loss_sq, sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(grads, m->g, sizeof(float) * m->np, cudaMemcpyDefault, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return mcuda(m, e, "ax_mlp_grad");
-  double acc = 0.0;
-  for (float v : part) acc += v;
-  *loss = (float)(0.5 * acc / ((double)M * kOut));
+  *loss = (float)(0.5 * sq / ((double)M * kOut));
   return gemm_status(m, "ax_mlp_grad");
 }
 
@@ -696,7 +788,7 @@ ax_status ax_mlp_train(ax_mlp *m, const void *X_bf16, const float *T, int64_t n_
   if (!m || !X_bf16 || !T || n_samples < batch || epochs < 1 || batch < 32 || batch % 32 || !(lr > 0.0f))
     return mfail(m, AX_EINVAL, "ax_mlp_train: bad arguments");
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = ensure_cap(m, batch);
+  cudaError_t e = ensure_grad_cap(m, batch);
   __nv_bfloat16 *Xb = nullptr;
   float *Tb = nullptr;
   int64_t *idx = nullptr;
@@ -705,7 +797,6 @@ ax_status ax_mlp_train(ax_mlp *m, const void *X_bf16, const float *T, int64_t n_
   if (e == cudaSuccess) e = cudaMalloc(&Tb, sizeof(float) * batch * kOut);
   if (e == cudaSuccess) e = cudaMalloc(&idx, sizeof(int64_t) * steps * batch);
   std::vector<int64_t> perm((size_t)n_samples);
-  std::vector<float> part(1024);
   SplitMix rng{seed};
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
@@ -722,11 +813,10 @@ ax_status ax_mlp_train(ax_mlp *m, const void *X_bf16, const float *T, int64_t n_
       adam<<<gfor(m->np), 256, 0, s>>>(m->np, m->p, m->g, m->am, m->av, lr, b1, b2, eps, c1, c2);
       e = refresh_bf16(m, s);
       if (e == cudaSuccess && (st == steps - 1)) {
-        e = cudaMemcpyAsync(part.data(), m->part, sizeof(float) * 1024, cudaMemcpyDeviceToHost, s);
+        double sq = 0.0;
+        e = cudaMemcpyAsync(&sq, m->loss_sq, sizeof(double), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        double acc = 0.0;
-        for (float v : part) acc += v;
-        ep_loss = 0.5 * acc / ((double)batch * kOut);
+        ep_loss = 0.5 * sq / ((double)batch * kOut);
       }
     }
     if (loss_history) loss_history[ep] = (float)ep_loss;
@@ -839,7 +929,7 @@ cudaError_t lp_apply(const ax_ctx *c, ax_mlp *m, LearnWork &W, double omega, boo
   const double *skip = W.S + kMlpSkip;
   if (scatter) lp_scatter<<<gfor(n), 256, 0, s>>>(n, W.r, P.off, P.idx, W.Ul);
   element_inputs<<<input_blocks(E), 32 * kInputWarps, 0, s>>>(E, nullptr, W.Ul, ax_ctx_vertices(c), W.F, W.scale, skip);
-  cudaError_t e = forward(m, W.F, E, s, skip);
+  cudaError_t e = forward(m, W.F, E, m->Y, s, skip);
   if (e != cudaSuccess) return e;
   lp_precond<<<kLpBlocks, red::kThreads, 0, s>>>(n, P.off, P.idx, m->Y, W.scale, W.dinv, W.r, W.w, P.mask,
                                                  (float)omega, W.z, W.part, W.cnt + 3, W.S);
@@ -1002,8 +1092,9 @@ void ax_mlp_destroy(ax_mlp *m) {
     cudaFree(m->Wb[l]);
     cudaFree(m->WTb[l]);
   }
-  cudaFree(m->Z1); cudaFree(m->Z2); cudaFree(m->Y); cudaFree(m->part);
-  cudaFree(m->H1); cudaFree(m->H2); cudaFree(m->dY); cudaFree(m->dZ1); cudaFree(m->dZ2); cudaFree(m->T1); cudaFree(m->T2);
+  cudaFree(m->Y); cudaFree(m->H1); cudaFree(m->H2);
+  cudaFree(m->Z1); cudaFree(m->Z2); cudaFree(m->sq); cudaFree(m->col); cudaFree(m->part); cudaFree(m->loss_sq);
+  cudaFree(m->dY); cudaFree(m->dZ1); cudaFree(m->dZ2);
   delete m;
 }
 
