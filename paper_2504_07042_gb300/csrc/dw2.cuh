@@ -58,33 +58,34 @@ struct acc2 {
   f2 s, c;
 };
 
-// The operand pair y of a product term, with its high parts negated (nh):
-// the products' rounding errors are then formed without a separate negation
-// (x.hi * (-y.hi) + p = -(x.hi * y.hi - p) exactly).
+// The operand pair y of a product term.
 struct opnd {
-  f2 h, l, nh;
+  f2 h, l;
 };
 
 // a = x * y (dw::mul_acc in each lane)
 __device__ __forceinline__ acc2 mul0(f2 xh, f2 xl, const opnd &y) {
   const f2 p = mul(xh, y.h);
-  const f2 np = mul(xh, y.nh);  // -p, exactly
-  f2 c = fma(xh, y.h, np);      // x.hi * y.hi - p
+  f2 c = fma(xh, y.h, mul(p, make_float2(-1.0f, -1.0f)));  // x.hi * y.hi - p
   c = fma(xh, y.l, c);
   c = fma(xl, y.h, c);
   return acc2{p, c};
 }
 
-// a += x * y (dw::mac in each lane)
+// a += x * y (dw::mac in each lane), with nbb = -(s - a.s) formed directly
+// (the negation of a rounded difference is exact).  The product is written as
+// a fused multiply-add onto +0: measured with this toolchain, a packed product
+// whose only use is a sum is contracted with that sum even in the form of
+// add() (then s = RN(a.s + x y) without the rounding that da and db account
+// for: errors of 2^-27), while the form here reproduces dw::mac bit for bit.
 __device__ __forceinline__ void mac(acc2 &a, f2 xh, f2 xl, const opnd &y) {
-  const f2 p = mul(xh, y.h);
-  const f2 npe = fma(xh, y.nh, p);  // -(x.hi * y.hi - p), exactly the negated error term
-  // TwoSum(a.s, p)
+  const f2 p = fma(xh, y.h, make_float2(0.0f, 0.0f));
   const f2 s = add(a.s, p);
-  const f2 bb = sub(s, a.s);
-  const f2 e = add(sub(a.s, sub(s, bb)), sub(p, bb));
+  const f2 nbb = sub(a.s, s);
+  const f2 da = sub(a.s, add(s, nbb));
+  const f2 db = fma(xh, y.h, nbb);
   a.s = s;
-  f2 c = add(a.c, sub(e, npe));  // a.c + (e + pe)
+  f2 c = add(a.c, add(da, db));
   c = fma(xh, y.l, c);
   a.c = fma(xl, y.h, c);
 }
@@ -105,7 +106,6 @@ __device__ __forceinline__ void contract(const float4 *__restrict__ eo2, const d
     const dw::dw o = dw::sub_lazy(in[m], in[N1 - 1 - m]);
     y[m].h = make_float2(e.hi, o.hi);
     y[m].l = make_float2(e.lo, o.lo);
-    y[m].nh = make_float2(-e.hi, -o.hi);
   }
 #pragma unroll
   for (int i = 0; i < c; ++i) {
