@@ -53,8 +53,6 @@ void release(ax_ctx *c) {
   cudaFree(c->c.lam);
   cudaFree(c->c.hx);
   cudaFree(c->c.hy);
-  cudaFree(c->c.wide);
-  c->c.wide = nullptr;
   cudaFree(c->c.kerr);
   c->c.kerr = nullptr;
   c->c.free_ws();
@@ -75,7 +73,6 @@ ax::AxArgs make_args(ax_ctx *c, const void *X, void *Y, void *stream) {
   a.kind = c->c.kind;
   a.geo = c->c.geo;
   a.lam = c->c.lam;
-  a.wide = c->c.wide;
   a.err = c->c.kerr;
   a.X = X;
   a.Y = Y;
@@ -224,11 +221,6 @@ ax_status ax_setup(ax_ctx **out, int64_t E, int N, const double *vertices, ax_ge
       // error word of the tensor-core kernel's bounded waits
       e = cudaMalloc(&c->c.kerr, sizeof(int));
       if (e == cudaSuccess) e = cudaMemsetAsync(c->c.kerr, 0, sizeof(int), s);
-    }
-    if (e == cudaSuccess && prec == AX_F64DW) {
-      // block list of the double-word kernel's scaled fix-up pass, zero at rest
-      e = cudaMalloc(&c->c.wide, (size_t)(E + 2) * sizeof(int));
-      if (e == cudaSuccess) e = cudaMemsetAsync(c->c.wide, 0, (size_t)(E + 2) * sizeof(int), s);
     }
     if (e == cudaSuccess) e = cudaMalloc(&flags, 4 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->vtx, vertices, (size_t)E * 24 * sizeof(double), cudaMemcpyDefault, s);

@@ -533,8 +533,8 @@ __device__ __forceinline__ int exp_field(float v) { return (__float_as_int(v) >>
 // element extents in [2^-20, 2^24] (checked at setup), values far below their
 // row's largest contribute below the accuracy, and X is converted by integer
 // instructions (dw::from_double_direct, whose range ends at 2^-74); Y goes
-// back the same way (dw::sum3_to_double_direct).  The fix-up kernel over the
-// other blocks converts on the FP64 pipe.
+// back the same way (dw::sum3_to_double_direct).  The other blocks are
+// converted on the FP64 pipe.
 __device__ __forceinline__ int mag_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
 __device__ __forceinline__ bool row_direct(int hmax) {
   return hmax == 0 || (hmax >= ((1023 - 60) << 20) && hmax < ((1023 + 61) << 20));
@@ -547,24 +547,19 @@ __device__ __forceinline__ bool row_direct(int hmax) {
 // pointer is 16-byte aligned, else consecutive words.  THREADS * N1 >= nvals.
 template <class P, int N1, int PITCH, int THREADS>
 __device__ __forceinline__ bool load_rows(const typename P::IO *__restrict__ src, int nvals, typename P::S *xs,
-                                          int tid, const int *emax) {
-  // emax (kScaleIO policies, or nullptr): per-element largest exponent field;
-  // each value is scaled by its element's power of two.  Without it the
-  // return value says whether a nonzero value lay outside the direct range.
+                                          int tid) {
+  // kScaleIO policies: returns whether a nonzero value lay outside the direct range
   using IO = typename P::IO;
   constexpr int n3 = N1 * N1 * N1, VEC = 16 / (int)sizeof(IO);
   bool wide = false;
   auto put = [&](int m, IO v) {
     const int row = m / N1;
     if constexpr (P::kScaleIO) {
-      if (emax) v = v * pow2i(io_shift(emax[m / n3]));
-    }
-    if constexpr (P::kScaleIO) {
       // each value alone is its own "row" here (a nonzero value is then at
       // least 2^-60: inside from_io_direct's range)
-      if (!emax) wide |= !row_direct(mag_hi(v));
+      wide |= !row_direct(mag_hi(v));
     }
-    xs[row * PITCH + (m - row * N1)] = P::st(emax ? P::from_io(v) : P::from_io_direct(v));
+    xs[row * PITCH + (m - row * N1)] = P::st(P::from_io_direct(v));
   };
   if constexpr (n3 % VEC == 0) {
     if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
@@ -625,11 +620,11 @@ struct FiberSmem {
   S *xs;        // [3][EPB][ES]: x, x0, x1; later t / Y_t, r / Y_r, s / Y_s
   S *sgeo;      // [EPB][GWD]: the elements' geometry records
   S *sax;       // [EPB][AXD]: per-element axis terms of the trilinear geometry (AXS)
-  int *sexp;    // [EPB] largest exponent field of each element's X (scaled fix-up pass)
+  int *sexp;    // kScaleIO: [EPB] largest exponent field of each element's X, then the block's flag
   __host__ __device__ static constexpr size_t a16(size_t b) { return (b + 15) / 16 * 16; }
   // all four carved from one 16-byte aligned buffer of `bytes` bytes
   static constexpr size_t bytes = a16(sizeof(S) * 3 * Sh::EPB * Sh::ES) + a16(sizeof(S) * Sh::EPB * GWD) +
-                                  a16(sizeof(S) * Sh::EPB * AXD) + a16(sizeof(int) * Sh::EPB);
+                                  a16(sizeof(S) * Sh::EPB * AXD) + a16(sizeof(int) * (Sh::EPB + 1));
   __device__ static __forceinline__ FiberSmem carve(unsigned char *raw) {
     FiberSmem m;
     m.xs = (S *)raw;
@@ -651,8 +646,8 @@ struct FiberSmem {
 // threads than the order's shape (a CTA shaped for several orders); those
 // threads only take part in the barriers.
 // ---------------------------------------------------------------------------
-template <class P, int N1, int KIND, int EM, bool IDLE, int SCALE, class XS, int EPB0 = kEpb<P, N1, KIND>>
-__device__ __forceinline__ bool fiber_block(const FiberSmem<P, N1, KIND, EM, EPB0> &sm, const int tid, const int64_t e0,
+template <class P, int N1, int KIND, int EM, bool IDLE, class XS, int EPB0 = kEpb<P, N1, KIND>>
+__device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB0> &sm, const int tid, const int64_t e0,
                                             const int nel, const typename P::S *__restrict__ geo,
                                             const typename P::S *__restrict__ lam, const XS &X,
                                             typename P::IO *__restrict__ Y) {
@@ -663,7 +658,6 @@ __device__ __forceinline__ bool fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   constexpr int n3 = Sh::n3, EPB = Sh::EPB, ES = Sh::ES;
   constexpr int GW = GeoWords<KIND>::value;
   static_assert(!IDLE || !P::kRoll, "idle threads are handled in the short (native) kernel body");
-  static_assert(SCALE == 0 || P::kScaleIO, "X scaling belongs to the policies with kScaleIO");
   S *const xs = sm.xs;          // [EPB][ES]: x, later Y
   S *const b0 = xs + EPB * ES;  // x0, later r
   S *const b1 = b0 + EPB * ES;  // x1, later s
@@ -698,63 +692,65 @@ __device__ __forceinline__ bool fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   // (a gathered X, X[m] = u[gid[m]], is read one row per thread)
   constexpr bool kRowsCoalesced =
       XS::kDirect && ((sizeof(typename P::IO) == 4 && (N1 == 2 || N1 == 4 || N1 == 8)) || (P::kRoll && N1 == 16));
-  // Policies with kScaleIO (float64 data in float32 pairs) run in two modes.
-  // SCALE = 1, the main kernel: X is converted directly and the block
-  // reports whether a row's largest magnitude lies outside the direct range
-  // (row_direct).  SCALE = 2, a fix-up kernel over only the reported blocks:
-  // each element's X is scaled by the power of two that brings its largest
-  // magnitude into [1, 2) before the conversion, and its Y is scaled back.
-  bool wide = false;  // SCALE 1: a row of this thread lies outside the direct range
-  int xshift = 0;     // SCALE 2: this thread's element entered as X * 2^xshift
-  if constexpr (SCALE == 2) {
-    if (live) {
-      const int64_t srow = e * n3 + q * N1;  // row q of element z
-      int mx = 0;
-#pragma unroll
-      for (int i = 0; i < N1; ++i) mx = max(mx, exp_field(X[srow + i]));
-      atomicMax(&sexp[z], mx);
-    }
-    __syncthreads();
-    if (live) xshift = io_shift(sexp[z]);
-  }
+  // Policies with kScaleIO (float64 data in float32 pairs): X is converted
+  // directly, and the threads test whether a row's largest magnitude lies
+  // outside the direct range (row_direct).  If any row of the block does, the
+  // block reads X again: each element is scaled by the power of two that
+  // brings its largest magnitude into [1, 2) before the conversion, and its Y
+  // is scaled back on the way out.  (As a second kernel over a list of such
+  // blocks this cost every call a launch, 4 us with an empty list: order 7,
+  // 512 elements 18.4 -> 14.3 us per call; 131072 elements unchanged.)
+  bool wide = false;  // a row of this thread lies outside the direct range
   if (act) {
     using IO = typename P::IO;
     if constexpr (kRowsCoalesced) {
-      wide = load_rows<P, N1, Sh::P, Sh::threads>(X.p + e0 * n3, nel * n3, xs, tid, SCALE == 2 ? sexp : nullptr);
+      wide = load_rows<P, N1, Sh::P, Sh::threads>(X.p + e0 * n3, nel * n3, xs, tid);
     } else {
       for (int row = tid; row < nel * N1 * N1; row += Sh::threads) {
         const int64_t src = e0 * n3 + (int64_t)row * N1;
         S *dst = xs + row * Sh::P;
-        // SCALE 2: one row per thread (threads = EPB N1^2), row tid of element z
-        const IO sc = SCALE == 2 ? (IO)pow2i(xshift) : IO(1);
-        int hmax = 0;       // SCALE 1: the row's largest magnitude (upper 32 bits)
-        bool tiny = false;  // SCALE 1: a nonzero value below from_io_direct's range
+        int hmax = 0;       // the row's largest magnitude (upper 32 bits)
+        bool tiny = false;  // a nonzero value below from_io_direct's range
 #pragma unroll
         for (int i = 0; i < N1; ++i) {
           const IO v = X[src + i];
-          if constexpr (SCALE == 1) {
+          if constexpr (P::kScaleIO) {
             hmax = max(hmax, mag_hi(v));
-            if constexpr (P::kScaleIO) tiny |= dw::tiny_nonzero((unsigned)mag_hi(v));
-            dst[i] = P::st(P::from_io_direct(v));
-          } else {
-            dst[i] = P::st(P::from_io(SCALE == 2 ? v * sc : v));
+            tiny |= dw::tiny_nonzero((unsigned)mag_hi(v));
           }
+          dst[i] = P::st(P::from_io_direct(v));
         }
-        if constexpr (SCALE == 1) wide |= tiny || !row_direct(hmax);
+        if constexpr (P::kScaleIO) wide |= tiny || !row_direct(hmax);
       }
     }
     if constexpr (GW > 0) {
       for (int m = tid; m < nel * GW; m += Sh::threads) sm.sgeo[(m / GW) * Buf::GWD + m % GW] = geo[e0 * GW + m];
     }
   }
-  bool any_wide = false;
-  if constexpr (SCALE == 1) {
-    any_wide = __syncthreads_or(wide);
+  if constexpr (P::kScaleIO) {
+    const bool any_wide = __syncthreads_or(wide);
+    if (tid == 0) sexp[EPB] = any_wide;  // read again when Y is stored (a register less meanwhile)
+    if (any_wide) {
+      if (tid < EPB) sexp[tid] = 0;
+      __syncthreads();
+      const int64_t srow = e * n3 + q * N1;  // row q of element z
+      if (live) {
+        int mx = 0;
+#pragma unroll 1
+        for (int i = 0; i < N1; ++i) mx = max(mx, exp_field(X[srow + i]));
+        atomicMax(&sexp[z], mx);
+      }
+      __syncthreads();
+      if (live) {
+        const typename P::IO sc = pow2i(io_shift(sexp[z]));
+        S *dst = xs + (z * N1 * N1 + q) * Sh::P;
+#pragma unroll 1
+        for (int i = 0; i < N1; ++i) dst[i] = P::st(P::from_io(X[srow + i] * sc));
+      }
+      __syncthreads();
+    }
   } else {
     __syncthreads();
-  }
-  if constexpr (SCALE == 2) {
-    if (tid < EPB) sexp[tid] = 0;  // every read of sexp came before the barrier
   }
   if constexpr (AXS) {
     // threads q < 2 N1 of each element: the N1 r-axis and N1 s-axis terms,
@@ -840,19 +836,20 @@ __device__ __forceinline__ bool fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     __syncthreads();  // every Y_r, Y_s value is in B0, B1
     if (live) {
       typename P::IO *ye = Y + e * n3 + qa + N1 * qb;
+      auto yt_of = [&](int k) { return kYtRegs ? yt[kYtRegs ? k : 0] : P::ld(x_e + ft + k * str_t); };
+      if (!sexp[EPB]) {
 #pragma unroll
-      for (int k = 0; k < N1; ++k) {
-        const int sidx = ft + k * str_t;
-        const V ytk = kYtRegs ? yt[kYtRegs ? k : 0] : P::ld(x_e + sidx);
-        const V yr = P::ld(r_e + sidx), ys = P::ld(s_e + sidx);
-        ye[k * N1 * N1] = SCALE == 1 ? P::sum3_io_direct(ytk, yr, ys) : P::sum3_io(ytk, yr, ys);
-      }
-      if constexpr (SCALE == 2) {
-        // undo the element's input shift on the values just stored (exact)
-        if (xshift != 0) {
-          const typename P::IO ysc = (typename P::IO)pow2i(-xshift);
-#pragma unroll 1
-          for (int k = 0; k < N1; ++k) ye[k * N1 * N1] *= ysc;
+        for (int k = 0; k < N1; ++k) {
+          const int sidx = ft + k * str_t;
+          ye[k * N1 * N1] = P::sum3_io_direct(yt_of(k), P::ld(r_e + sidx), P::ld(s_e + sidx));
+        }
+      } else {
+        // the element entered as X 2^d: undo it (exact)
+        const typename P::IO ysc = pow2i(-io_shift(sexp[z]));
+#pragma unroll
+        for (int k = 0; k < N1; ++k) {
+          const int sidx = ft + k * str_t;
+          ye[k * N1 * N1] = P::sum3_io(yt_of(k), P::ld(r_e + sidx), P::ld(s_e + sidx)) * ysc;
         }
       }
     }
@@ -878,9 +875,9 @@ __device__ __forceinline__ bool fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     if (act) {
       const int i = qa, j = qb;
       Geometry<P, N1, KIND> gm;
-      gm.template prologue<AXS>(sgeo_z, cx, cw, i, j,
-                                (KIND == AX_GEOM_STORED && live) ? geo + e * 7 * n3 : nullptr,
-                                (KIND == AX_GEOM_TRILINEAR_PARTIAL && live) ? lam + e * n3 : nullptr, sax_z);
+      const int64_t eg = live ? e : e0;
+      gm.template prologue<AXS>(sgeo_z, cx, cw, i, j, KIND == AX_GEOM_STORED ? geo + eg * 7 * n3 : nullptr,
+                                KIND == AX_GEOM_TRILINEAR_PARTIAL ? lam + eg * n3 : nullptr, sax_z);
 #pragma unroll
       for (int k = 0; k < N1; ++k) {
         const int sidx = ft + k * str_t;
@@ -922,19 +919,16 @@ __device__ __forceinline__ bool fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   }
 
   __syncthreads();  // the next block reuses the shared buffers
-  return any_wide;
 }
 
 // ---------------------------------------------------------------------------
 // the per-order kernel: blocks of EPB elements, persistent over blocks when
 // the grid is capped (autotuner)
 // ---------------------------------------------------------------------------
-// wide: kScaleIO policies: list of the blocks whose X left the direct range
-// ([0] count, [1] exit counter of the fix-up kernel, [2..] block indices).
 template <class P, int N1, int KIND, int EM>
 __global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads, kMinCtas<P, N1, KIND>)
     ax_fiber_kernel(int64_t E, const typename P::S *__restrict__ geo, const typename P::S *__restrict__ lam,
-                    const typename P::IO *__restrict__ X, typename P::IO *__restrict__ Y, int *__restrict__ wide) {
+                    const typename P::IO *__restrict__ X, typename P::IO *__restrict__ Y) {
   using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
   using Buf = FiberSmem<P, N1, KIND, EM>;
   using S = typename P::S;
@@ -942,58 +936,18 @@ __global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads, kMi
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ S sgeo[EPB][Buf::GWD];
   __shared__ S sax[Buf::AXS ? EPB : 1][Buf::AXD];
-  Buf sm;
-  sm.xs = (S *)smem_raw;
-  sm.sgeo = &sgeo[0][0];
-  sm.sax = &sax[0][0];
-  sm.sexp = nullptr;
-  const int tid = threadIdx.x;
-  const int64_t nblk = (E + EPB - 1) / EPB;
-  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-    const int64_t e0 = blk * EPB;
-    const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
-    const bool w = fiber_block<P, N1, KIND, EM, false, P::kScaleIO ? 1 : 0>(sm, tid, e0, nel, geo, lam,
-                                                                           XDirect<typename P::IO>{X}, Y);
-    if constexpr (P::kScaleIO) {
-      if (w && tid == 0) wide[2 + atomicAdd(&wide[0], 1)] = (int)blk;
-    }
-  }
-}
-
-// The fix-up kernel of the kScaleIO policies: the listed blocks again, with X
-// scaled per element; the last CTA to finish clears the list.
-template <class P, int N1, int KIND, int EM>
-__global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads)
-    ax_fiber_fix_kernel(int64_t E, const typename P::S *__restrict__ geo, const typename P::S *__restrict__ lam,
-                        const typename P::IO *__restrict__ X, typename P::IO *__restrict__ Y, int *__restrict__ wide) {
-  using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
-  using Buf = FiberSmem<P, N1, KIND, EM>;
-  using S = typename P::S;
-  constexpr int EPB = Sh::EPB;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ S sgeo[EPB][Buf::GWD];
-  __shared__ S sax[Buf::AXS ? EPB : 1][Buf::AXD];
-  __shared__ int sexp[EPB];
+  __shared__ int sexp[P::kScaleIO ? EPB + 1 : 1];
   Buf sm;
   sm.xs = (S *)smem_raw;
   sm.sgeo = &sgeo[0][0];
   sm.sax = &sax[0][0];
   sm.sexp = sexp;
   const int tid = threadIdx.x;
-  if (tid < EPB) sexp[tid] = 0;
-  __syncthreads();
-  const int cnt = *(volatile int *)&wide[0];
-  for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
-    const int64_t e0 = (int64_t)wide[2 + i] * EPB;
+  const int64_t nblk = (E + EPB - 1) / EPB;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    const int64_t e0 = blk * EPB;
     const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
-    fiber_block<P, N1, KIND, EM, false, 2>(sm, tid, e0, nel, geo, lam, XDirect<typename P::IO>{X}, Y);
-  }
-  if (tid == 0) {
-    __threadfence();
-    if (atomicAdd(&wide[1], 1) == (int)gridDim.x - 1) {
-      wide[0] = 0;
-      wide[1] = 0;
-    }
+    fiber_block<P, N1, KIND, EM, false>(sm, tid, e0, nel, geo, lam, XDirect<typename P::IO>{X}, Y);
   }
 }
 
@@ -1033,31 +987,19 @@ __global__ void __launch_bounds__(Shape<N1, 1, kEpb<P, N1, KIND>>::threads)
   }
 }
 
-// CTAs of the fix-up kernel (a persistent loop over the listed blocks)
-constexpr int64_t kFixGrid = 256;
-
+// Dynamic shared memory of a kernel of this shape.
 template <class P, int N1, int KIND, int EM>
-cudaError_t launch_ax_em(const AxArgs &a) {
+size_t launch_smem(const void *kernel) {
   using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
-  const int64_t nblk = (a.E + Sh::EPB - 1) / Sh::EPB;
-  if (nblk <= 0) return cudaSuccess;
-  int64_t grid = a.grid > 0 && a.grid < nblk ? a.grid : nblk;
-  if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  size_t smem = (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S);
+  const size_t smem = (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S);
   if constexpr (P::kTargetWarpsPerSM > 0 && N1 == 8 &&
                 (KIND == AX_GEOM_TRILINEAR || KIND == AX_GEOM_TRILINEAR_PARTIAL)) {
     // cap the resident CTAs by their shared memory (the kernel uses only its share)
-    static int sm_smem = 0;
-    if (!sm_smem) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    }
-    static int static_smem = -1;
-    if (static_smem < 0) {
-      cudaFuncAttributes fa;
-      static_smem = cudaFuncGetAttributes(&fa, ax_fiber_kernel<P, N1, KIND, EM>) == cudaSuccess ? (int)fa.sharedSizeBytes : 4096;
-    }
+    int dev = 0, sm_smem = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaFuncAttributes fa;
+    const int static_smem = cudaFuncGetAttributes(&fa, kernel) == cudaSuccess ? (int)fa.sharedSizeBytes : 4096;
     const int warps = (Sh::threads + 31) / 32;
     int ctas = (P::kTargetWarpsPerSM + warps / 2) / warps;
     if (ctas < 1) ctas = 1;
@@ -1065,8 +1007,19 @@ cudaError_t launch_ax_em(const AxArgs &a) {
     // reserves, with 1 KB to spare (with none the driver chose a smaller
     // shared-memory carveout and only ctas - 1 CTAs fitted: measured)
     const size_t cap = sm_smem > 0 ? (size_t)sm_smem / ctas - (size_t)static_smem - 2048 : 0;
-    if (cap > smem && cap <= 200 * 1024) smem = cap;
+    if (cap > smem && cap <= 200 * 1024) return cap;
   }
+  return smem;
+}
+
+template <class P, int N1, int KIND, int EM>
+cudaError_t launch_ax_em(const AxArgs &a) {
+  using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
+  const int64_t nblk = (a.E + Sh::EPB - 1) / Sh::EPB;
+  if (nblk <= 0) return cudaSuccess;
+  const int64_t grid = a.grid > 0 && a.grid < nblk ? a.grid : nblk;
+  if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+  static const size_t smem = launch_smem<P, N1, KIND, EM>((const void *)ax_fiber_kernel<P, N1, KIND, EM>);
   // per instantiation; static shared memory counts against the same 48 KB
   // default, so the attribute is set whatever the dynamic size
   static bool attr_set = false;
@@ -1076,25 +1029,9 @@ cudaError_t launch_ax_em(const AxArgs &a) {
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  if (P::kScaleIO && !a.wide) return cudaErrorInvalidValue;  // the context's block list is required
   ax_fiber_kernel<P, N1, KIND, EM><<<(unsigned)grid, Sh::threads, smem, a.stream>>>(
       a.E, (const typename P::S *)a.geo, (const typename P::S *)a.lam, (const typename P::IO *)a.X,
-      (typename P::IO *)a.Y, a.wide);
-  if constexpr (P::kScaleIO) {
-    // the blocks whose X left the direct range, again with scaling (usually none)
-    static bool fix_attr = false;
-    const size_t fsmem = (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S);
-    if (!fix_attr) {
-      cudaError_t e = cudaFuncSetAttribute(ax_fiber_fix_kernel<P, N1, KIND, EM>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
-      if (e != cudaSuccess) return e;
-      fix_attr = true;
-    }
-    const int64_t fgrid = nblk < kFixGrid ? nblk : kFixGrid;
-    ax_fiber_fix_kernel<P, N1, KIND, EM><<<(unsigned)fgrid, Sh::threads, fsmem, a.stream>>>(
-        a.E, (const typename P::S *)a.geo, (const typename P::S *)a.lam, (const typename P::IO *)a.X,
-        (typename P::IO *)a.Y, a.wide);
-  }
+      (typename P::IO *)a.Y);
   return cudaGetLastError();
 }
 

@@ -50,7 +50,6 @@ struct Ctx {
   size_t geo_bytes = 0;
   void *lam = nullptr;
   size_t lam_bytes = 0;
-  int *wide = nullptr;  // AX_F64DW: block list of the scaled fix-up pass (int[2 + E], zeroed)
   int *kerr = nullptr;  // AX_TF32: error word of the tensor-core AxLocal's bounded waits
   // device staging buffers for ax_local_host
   void *hx = nullptr, *hy = nullptr;
@@ -87,9 +86,6 @@ struct AxArgs {
   cudaStream_t stream = nullptr;
   int tile = 0;      // tile variant (elements per CTA: 0 = base, 1 = twice; FP32 only)
   int64_t grid = 0;  // CTAs to launch (0 = one per block of elements; fewer = persistent loop)
-  // double-word precision: the context's list of element blocks whose X left
-  // the kernel's direct range (int[2 + E], zero at rest; see ax_fiber.cuh)
-  int *wide = nullptr;
   // kernels with bounded waits (tensor-core AxLocal): error word, nonzero
   // once a wait ran out (read by the context's synchronising calls)
   int *err = nullptr;

@@ -139,10 +139,10 @@ __device__ __noinline__ void ax_tile(unsigned char *smem, const Group &g, int64_
   for (int64_t b = e0; b < e0 + cnt; b += Sh::EPB) {
     const int nel = (int)((e0 + cnt - b) < Sh::EPB ? (e0 + cnt - b) : Sh::EPB);
     if constexpr (PCG) {
-      fiber::fiber_block<P, N1, KIND, 1, true, 0, fiber::XGather<float>, 0>(
+      fiber::fiber_block<P, N1, KIND, 1, true, fiber::XGather<float>, 0>(
           sm, tid, b, nel, (const float *)g.geo, (const float *)g.lam, fiber::XGather<float>{p, gid + g.loc}, Yg);
     } else {
-      fiber::fiber_block<P, N1, KIND, 1, true, 0, fiber::XDirect<float>, 0>(
+      fiber::fiber_block<P, N1, KIND, 1, true, fiber::XDirect<float>, 0>(
           sm, tid, b, nel, (const float *)g.geo, (const float *)g.lam, fiber::XDirect<float>{X + g.loc}, Yg);
     }
   }
