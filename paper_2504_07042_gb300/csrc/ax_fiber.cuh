@@ -34,6 +34,15 @@
 namespace ax {
 namespace fiber {
 
+// 1-ulp reciprocal of a normal float whose reciprocal is normal too: the
+// determinants of elements inside the extents that setup accepts (a general
+// fast division also tests for divisors above 2^126, three more instructions)
+__device__ __forceinline__ float rcp32(float b) {
+  float v;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(b));
+  return v;
+}
+
 // ---------------------------------------------------------------------------
 // arithmetic policies
 // ---------------------------------------------------------------------------
@@ -72,7 +81,7 @@ struct Native {
   __device__ static __forceinline__ IO sum3_io_direct(V a, V b, V c) { return (a + b) + c; }
   __device__ static __forceinline__ V div(V a, V b) {
     if constexpr (sizeof(T) == 4)
-      return __fdividef(a, b);  // 2-ulp quotient: the FP32 path's tolerance is 2e-5
+      return a * rcp32(b);  // 2-ulp quotient: the FP32 path's tolerance is 2e-5
     else
       return a / b;
   }
@@ -249,7 +258,8 @@ __host__ __device__ constexpr int pick_epb(int F) {
 // SM); bounded to five CTAs (96 registers, no spills) it runs 2.4% faster.
 // FP32 (40-64 registers, mostly faster as they are): N = 5 partial 4
 // elements (153 -> 163), N = 9 parallelepiped 2 (243 -> 251), N = 11 stored
-// 1 element, 4 CTAs (156 -> 172); N1 = 16 two CTAs (the packed fiber
+// 1 element, 4 CTAs (156 -> 172); N = 7 trilinear eight CTAs (64 registers
+// instead of 68: 298 -> 304); N1 = 16 two CTAs (the packed fiber
 // product, kPairedF32, would otherwise take 161 registers).
 __host__ __device__ constexpr int shape_epb(int pc, int N1, int KIND) {
   return pc == 0 ? (N1 == 6    ? (KIND == AX_GEOM_TRILINEAR ? 7 : KIND == AX_GEOM_TRILINEAR_PARTIAL ? 6 : 0)
@@ -264,6 +274,7 @@ __host__ __device__ constexpr int shape_min_ctas(int pc, int N1, int KIND) {
                     : N1 == 6  ? (KIND == AX_GEOM_TRILINEAR ? 3 : KIND == AX_GEOM_TRILINEAR_PARTIAL ? 4 : 0)
                     : N1 == 10 ? (KIND == AX_GEOM_TRILINEAR ? 5 : KIND == AX_GEOM_TRILINEAR_PARTIAL ? 2 : 0)
                                : 0)
+                 : (N1 == 8 && KIND == AX_GEOM_TRILINEAR)  ? 8
                  : (N1 == 12 && KIND == AX_GEOM_STORED) ? 4
                  : N1 == 16                              ? 2
                                                         : 0;
@@ -277,7 +288,6 @@ constexpr int kShapeClass = P::kRoll ? 0 : sizeof(typename P::S) == 4 ? 1 : -1;
 // kinds in 8-byte arithmetic (double-word, FP64) and for every recompute
 // kind at N1 = 6; the stored and parallelepiped kinds elsewhere, and FP32
 // at N1 = 10, 12, run faster with the smaller CTAs (more of them per SM).
-// The exceptions of shape_epb come first.
 template <class P, int N1, int KIND>
 constexpr int kEpb =
     (kShapeClass<P> >= 0 && shape_epb(kShapeClass<P>, N1, KIND)) ? shape_epb(kShapeClass<P>, N1, KIND)
@@ -310,16 +320,88 @@ template <class P, int N1, int KIND>
 constexpr bool kShareAxis = (KIND == AX_GEOM_TRILINEAR || KIND == AX_GEOM_TRILINEAR_PARTIAL) &&
                             (P::kRoll ? N1 <= 6 : sizeof(typename P::V) == 8);
 
-template <int N1, int EM = 1, int EPB0 = 0>
+// An element in shared memory: node (i, j, k) at i + P j + PK k, in words.
+// 8-byte words (double-word, FP64: bound by their pipes): rows padded
+// by one word.  4-byte words: the float32 kernels move about 15 words per node
+// through shared memory and are bound by it next to issue, so their pitches
+// come from a search over a model of the banks (32 of 4 bytes, vectors of 2
+// and 4 words served in phases of 16 and 8 lanes) for the fewest wavefronts of
+// a node's accesses: four by r-fiber owners (lane (j, k), a row each, in
+// vectors of `vec` words where that costs no more), four by s-fiber owners
+// (lane (i, k)), seven by t-fiber owners (lane (i, j)).  15 is the least;
+// padded rows alone need 22 at N1 = 4, 8 and 16, 23 to 28 at 6, 9, 10 and 12
+// to 14, 34 to 77 at 5, 7, 11 and 15.  Together with the loads below and the
+// packed geometry (Geometry2), measured on GB300: order 7 trilinear 258 -> 221
+// us for 131072 elements, order 5 stored 421 -> 366 us for 148877, 1.02 to 1.47
+// times at every order and kind of 3.2e7 nodes but the stored kind at order 1
+// (0.98).
+struct Pitches {
+  int P, PK, ES, vec;  // row, plane and element pitch; words per row access
+};
+//                                    wavefronts per node: N1 = 3: 23, 4: 19, 5: 23, 6: 20.5, 7: 21, 8: 15, 9: 17.7,
+constexpr Pitches kPitches32[17] = {  // 10: 17.5, 11: 19, 12: 15.8, 13: 18.3, 14: 18.1, 15: 22, 16: 15
+    {}, {}, {2, 6, 12, 2}, {3, 11, 41, 1}, {4, 20, 80, 4}, {5, 25, 153, 1}, {6, 36, 228, 2}, {7, 52, 369, 1},
+    {12, 104, 820, 4}, {9, 81, 729, 1}, {10, 106, 1054, 2}, {11, 121, 1331, 1}, {12, 172, 2036, 4}, {13, 169, 2197, 1},
+    {14, 206, 2874, 2}, {15, 225, 3375, 1}, {20, 336, 5356, 4}};
+// kinds of layout: padded rows, for words of any size, or the searched one
+enum { kPaddedRows = 0, kSearched32 = 1 };
+template <class P, int N1, int KIND>
+constexpr int kLayout = sizeof(typename P::S) == 4 && !(N1 == 8 && KIND == AX_GEOM_STORED) ? kSearched32 : kPaddedRows;
+template <int N1, int LK>
+struct Layout {
+  static constexpr Pitches pt =
+      LK == kSearched32 ? kPitches32[N1] : Pitches{N1 + 1, N1 * (N1 + 1), N1 * N1 * (N1 + 1), 1};
+  static constexpr int P = pt.P, PK = pt.PK, ES = pt.ES, vec = pt.vec;
+  static_assert(P >= N1 && PK >= (N1 - 1) * P + N1 && ES >= (N1 - 1) * (PK + P) + N1, "nodes apart");
+  static_assert(N1 % vec == 0 && P % vec == 0 && PK % vec == 0 && ES % vec == 0, "aligned rows");
+  // row j of the t-fibers owned by threads N1 b .. N1 b + N1 - 1: where a row
+  // fills whole banks (N1 = 8, 16) a warp takes rows that lie 8 or 16 banks
+  // apart (not in the stored kind at N1 = 8, whose factors a warp then reads
+  // in 32-byte pieces: it is bound by HBM, 180 against 168 GDOF/s)
+  __host__ __device__ static constexpr int row_of(int b) {
+    return LK == kSearched32 && N1 == 8    ? ((b & 3) << 1) | (b >> 2)                          // 0 2 4 6 | 1 3 5 7
+           : LK == kSearched32 && N1 == 16 ? ((b >> 1) & 3) | ((b & 1) << 2) | ((b >> 3) << 3)  // 0 4 | 1 5 | 2 6 | ..
+                                           : b;
+  }
+};
+
+template <int N1, int EM = 1, int EPB0 = 0, int LK = kPaddedRows>
 struct Shape {
+  using L = Layout<N1, LK>;
   static constexpr int n3 = N1 * N1 * N1;
   static constexpr int F = N1 * N1;  // fibers (threads) per element
   static constexpr int EPB = EM * (EPB0 > 0 ? EPB0 : (F >= 128 ? 1 : 128 / F));  // elements per CTA (EM: tile variant)
   static constexpr int threads = F * EPB;
-  static constexpr int P = N1 + 1;            // padded row
-  static constexpr int ES = N1 * N1 * P;      // padded element size (words)
-  __device__ static __forceinline__ int at(int i, int j, int k) { return i + P * (j + N1 * k); }
+  static constexpr int P = L::P, PK = L::PK, ES = L::ES;  // row, plane and element pitch (words)
+  __device__ static __forceinline__ int at(int i, int j, int k) {
+    return LK == kPaddedRows ? i + P * (j + N1 * k) : i + P * j + PK * k;
+  }
 };
+
+// a row of N values in vectors of VEC floats
+template <int N, int VEC>
+__device__ __forceinline__ void load_row(const float *p, float v[N]) {
+#pragma unroll
+  for (int c = 0; c < N; c += VEC) {
+    if constexpr (VEC == 4) {
+      const float4 t = *reinterpret_cast<const float4 *>(p + c);
+      v[c] = t.x; v[c + 1] = t.y; v[c + 2] = t.z; v[c + 3] = t.w;
+    } else {
+      const float2 t = *reinterpret_cast<const float2 *>(p + c);
+      v[c] = t.x; v[c + 1] = t.y;
+    }
+  }
+}
+template <int N, int VEC>
+__device__ __forceinline__ void store_row(float *p, const float v[N]) {
+#pragma unroll
+  for (int c = 0; c < N; c += VEC) {
+    if constexpr (VEC == 4)
+      *reinterpret_cast<float4 *>(p + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+    else
+      *reinterpret_cast<float2 *>(p + c) = make_float2(v[c], v[c + 1]);
+  }
+}
 
 // ---------------------------------------------------------------------------
 // geometry (getFactors of Algorithm 4) in policy arithmetic
@@ -510,6 +592,98 @@ struct Geometry {
 };
 
 
+// The float32 geometry at two nodes of a fiber at once, the nodes k and N - k
+// in the lanes of packed FP32x2 instructions (dw2.cuh): the same operations in
+// the same order per node as Geometry<Native<float>>, half the instructions.
+// The coefficients along the fiber are held twice, once per lane: up to 17
+// more registers (kPackedGeo says where that pays).
+template <int N1, int KIND>
+struct Geometry2 {
+  using f2 = dw2::f2;
+  using G = Geometry<Native<float>, N1, KIND>;
+  f2 k00[3], k01[3], k11[3], k02[2], k12[2], k22, dt[3], h[6];
+  const float *gl;
+  float wij;
+  __device__ __forceinline__ static f2 both(float v) { return make_float2(v, v); }
+  __device__ __forceinline__ explicit Geometry2(const G &g) : gl(g.gl), wij(g.wij) {
+    if constexpr (KIND == AX_GEOM_PARALLELEPIPED) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) h[q] = both(g.h[q]);
+    } else if constexpr (KIND != AX_GEOM_STORED) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        k00[q] = both(g.k00[q]);
+        k01[q] = both(g.k01[q]);
+        k11[q] = both(g.k11[q]);
+        if constexpr (KIND == AX_GEOM_TRILINEAR) dt[q] = both(g.dt[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        k02[q] = both(g.k02[q]);
+        k12[q] = both(g.k12[q]);
+      }
+      k22 = both(g.k22);
+    }
+  }
+  __device__ __forceinline__ static f2 quad(const f2 c[3], f2 t) { return dw2::fma(t, dw2::fma(t, c[2], c[1]), c[0]); }
+  __device__ __forceinline__ static f2 lin(const f2 c[2], f2 t) { return dw2::fma(t, c[1], c[0]); }
+  __device__ __forceinline__ static f2 neg(f2 a) { return make_float2(-a.x, -a.y); }
+  // a b + d e  (nc: one factor of the subtracted product, negated)
+  __device__ __forceinline__ static f2 det2n(f2 a, f2 b, f2 nc, f2 d) { return dw2::fma(nc, d, dw2::mul(a, b)); }
+  __device__ __forceinline__ static f2 dot(f2 a, f2 b, f2 c, const f2 y[3]) {
+    return dw2::fma(c, y[2], dw2::fma(b, y[1], dw2::mul(a, y[0])));
+  }
+  // (r, s, t) = G (x0, x1, x2) at local nodes l (lane 0, t = -tk... any pair) and l2 (lane 1)
+  __device__ __forceinline__ void apply(int l, int l2, f2 t, float wk, const f2 xv[3], f2 out[3]) const {
+    constexpr int n3 = N1 * N1 * N1;
+    f2 A[6], y[3];
+    if constexpr (KIND == AX_GEOM_STORED) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) A[q] = make_float2(gl[q * n3 + l], gl[q * n3 + l2]);
+      y[0] = xv[0]; y[1] = xv[1]; y[2] = xv[2];
+    } else if constexpr (KIND == AX_GEOM_PARALLELEPIPED) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) A[q] = h[q];
+      const f2 W = both(wij * wk);  // the weights of nodes k and N - k are equal
+      y[0] = dw2::mul(W, xv[0]); y[1] = dw2::mul(W, xv[1]); y[2] = dw2::mul(W, xv[2]);
+    } else {
+      const f2 K00 = quad(k00, t), K01 = quad(k01, t), K11 = quad(k11, t), K02 = lin(k02, t), K12 = lin(k12, t);
+      const f2 n01 = neg(K01), n02 = neg(K02), n12 = neg(K12);
+      A[0] = det2n(K11, k22, n12, K12);
+      A[1] = det2n(K02, K12, n01, k22);
+      A[2] = det2n(K01, K12, n02, K11);
+      A[3] = det2n(K00, k22, n02, K02);
+      A[4] = det2n(K01, K02, n12, K00);
+      A[5] = det2n(K00, K11, n01, K01);
+      f2 lam;
+      if constexpr (KIND == AX_GEOM_TRILINEAR) {
+        const f2 det = quad(dt, t);
+        lam = dw2::mul(both(wij * wk), make_float2(rcp32(det.x), rcp32(det.y)));
+      } else {
+        lam = make_float2(gl[l], gl[l2]);
+      }
+      y[0] = dw2::mul(lam, xv[0]); y[1] = dw2::mul(lam, xv[1]); y[2] = dw2::mul(lam, xv[2]);
+    }
+    out[0] = dot(A[0], A[1], A[2], y);
+    out[1] = dot(A[1], A[3], A[4], y);
+    out[2] = dot(A[2], A[4], A[5], y);
+  }
+};
+// Where the float32 kernels take it.  Measured on GB300 (3.2e7 nodes, GDOF/s,
+// packed / one node at a time, same layouts): trilinear faster at every order
+// but N = 5 (equal), N = 3 221 / 193, 7 272 / 264, 14 187 / 174; the partial
+// kind at N = 7 242 / 202, 11 225 / 196, slower at N <= 5 (183 / 205 at 5) and
+// at 8; the stored and parallelepiped kinds, whose node is short, within 4%
+// from N = 5 on and slower below or where the registers cost CTAs (stored:
+// 175 / 192 at N = 10), but for stored at N = 3 and 8 (183 / 167, 165 / 133).
+template <class P, int N1, int KIND>
+constexpr bool kPackedGeo = !P::kRoll && sizeof(typename P::V) == 4 &&
+                            (KIND == AX_GEOM_TRILINEAR              ? true
+                             : KIND == AX_GEOM_TRILINEAR_PARTIAL    ? N1 > 6 && N1 != 9
+                             : KIND == AX_GEOM_PARALLELEPIPED       ? N1 > 5 && N1 != 12
+                                                                    : N1 == 4 || N1 == 9);
+
+
 // Power-of-two scaling of an element's float64 values (policies with
 // kScaleIO).  emax is the largest biased exponent field among the element's
 // values; the shift d brings the largest magnitude into [1, 2) (clamped so
@@ -540,51 +714,14 @@ __device__ __forceinline__ bool row_direct(int hmax) {
   return hmax == 0 || (hmax >= ((1023 - 60) << 20) && hmax < ((1023 + 61) << 20));
 }
 
-// Coalesced copy of a block of values (contiguous in HBM) into padded
-// shared-memory rows of N1 values (pitch PITCH), converted by the policy P:
-// value m goes to row m / N1 at i = m % N1.  Consecutive threads read
-// consecutive 16-byte vectors when the values come in whole vectors and the
-// pointer is 16-byte aligned, else consecutive words.  THREADS * N1 >= nvals.
-template <class P, int N1, int PITCH, int THREADS>
-__device__ __forceinline__ bool load_rows(const typename P::IO *__restrict__ src, int nvals, typename P::S *xs,
-                                          int tid) {
-  // kScaleIO policies: returns whether a nonzero value lay outside the direct range
-  using IO = typename P::IO;
-  constexpr int n3 = N1 * N1 * N1, VEC = 16 / (int)sizeof(IO);
-  bool wide = false;
-  auto put = [&](int m, IO v) {
-    const int row = m / N1;
-    if constexpr (P::kScaleIO) {
-      // each value alone is its own "row" here (a nonzero value is then at
-      // least 2^-60: inside from_io_direct's range)
-      wide |= !row_direct(mag_hi(v));
-    }
-    xs[row * PITCH + (m - row * N1)] = P::st(P::from_io_direct(v));
-  };
-  if constexpr (n3 % VEC == 0) {
-    if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-      using VT = typename std::conditional<sizeof(IO) == 4, float4, double2>::type;
-      const VT *srcv = reinterpret_cast<const VT *>(src);
-#pragma unroll
-      for (int s = 0; s < (N1 + VEC - 1) / VEC; ++s) {
-        const int mv = tid + s * THREADS;
-        if (mv * VEC < nvals) {
-          const VT v = srcv[mv];
-          const IO *pv = reinterpret_cast<const IO *>(&v);
-#pragma unroll
-          for (int c = 0; c < VEC; ++c) put(mv * VEC + c, pv[c]);
-        }
-      }
-      return wide;
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < N1; ++s) {
-    const int m = tid + s * THREADS;
-    if (m < nvals) put(m, src[m]);
-  }
-  return wide;
-}
+// Double-word blocks that load one i-row per thread instead of the thread's
+// t-fiber.  Measured on GB300 (3.2e7 nodes): at N1 = 3, 12 and 14 the t-fibers
+// cost registers that the arithmetic needs (9% slower for the trilinear kind at
+// N1 = 3, 5 and 17% for the stored kind at 12 and 14); at the other orders they
+// are equal to 3%, or faster (N1 = 4 stored 80 against 58 GDOF/s, N1 = 16 by 5
+// to 9%).
+template <class P, int N1>
+constexpr bool kRowLoads = P::kRoll && (N1 == 3 || N1 == 12 || N1 == 14);
 
 template <int KIND>
 struct GeoWords {
@@ -596,13 +733,11 @@ struct GeoWords {
 // fused into the load).
 template <typename IO>
 struct XDirect {
-  static constexpr bool kDirect = true;
   const IO *__restrict__ p;
   __device__ __forceinline__ IO operator[](int64_t m) const { return p[m]; }
 };
 template <typename IO>
 struct XGather {
-  static constexpr bool kDirect = false;
   const IO *__restrict__ u;
   const gidx *__restrict__ gid;
   __device__ __forceinline__ IO operator[](int64_t m) const { return u[gid[m]]; }
@@ -612,7 +747,7 @@ struct XGather {
 // EPB0: the block shape (kEpb for the per-order kernels).
 template <class P, int N1, int KIND, int EM, int EPB0 = kEpb<P, N1, KIND>>
 struct FiberSmem {
-  using Sh = Shape<N1, EM, EPB0>;
+  using Sh = Shape<N1, EM, EPB0, kLayout<P, N1, KIND>>;
   using S = typename P::S;
   static constexpr int GW = GeoWords<KIND>::value, GWD = GW > 0 ? GW : 1;
   static constexpr bool AXS = kShareAxis<P, N1, KIND>;
@@ -651,11 +786,11 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
                                             const int nel, const typename P::S *__restrict__ geo,
                                             const typename P::S *__restrict__ lam, const XS &X,
                                             typename P::IO *__restrict__ Y) {
-  using Sh = Shape<N1, EM, EPB0>;
+  using Sh = Shape<N1, EM, EPB0, kLayout<P, N1, KIND>>;
   using Buf = FiberSmem<P, N1, KIND, EM, EPB0>;
   using V = typename P::V;
   using S = typename P::S;
-  constexpr int n3 = Sh::n3, EPB = Sh::EPB, ES = Sh::ES;
+  constexpr int n3 = Sh::n3, F = Sh::F, EPB = Sh::EPB, ES = Sh::ES;
   constexpr int GW = GeoWords<KIND>::value;
   static_assert(!IDLE || !P::kRoll, "idle threads are handled in the short (native) kernel body");
   S *const xs = sm.xs;          // [EPB][ES]: x, later Y
@@ -666,7 +801,8 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   constexpr int AXW = Geometry<P, N1, KIND>::kAxisWords;
   const bool act = !IDLE || tid < Sh::threads;
   const int z = tid / Sh::F, q = tid % Sh::F;
-  const int qa = q % N1, qb = q / N1;
+  const int qa = q % N1, qb = q / N1;   // this thread's r-fiber (j, k), s-fiber (i, k) and t-fiber (i, jt)
+  const int jt = Sh::L::row_of(qb);
   const typename P::C *eoD = c_eoD + tab_off_D(N1);
   const typename P::C *eoDT = c_eoDT + tab_off_D(N1);
   const float4 *eo2D = c_eo2D + tab_off_P(N1), *eo2DT = c_eo2DT + tab_off_P(N1);
@@ -677,53 +813,65 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   const int64_t e = e0 + z;
   const bool live = act && z < nel;
 
-  // pass 0: the CTA's elements (contiguous in HBM) into padded shared memory.
-  // Value m of the block sits in row m / N1 (row = j + N1 (k + N1 z) is also
-  // the padded row index) at i = m % N1.  Float32 data at N1 = 2, 4, 8 and
-  // double-word data at N1 = 16 are read coalesced (load_rows): measured on
-  // GB300 4-16% faster than one row per thread for float32 at N = 3 and 7,
-  // 3-10% for double-word at N = 15.  Elsewhere one i-row of N1 values per
-  // thread: the coalesced form measured 10% slower for float32 N = 5 and 29%
-  // for double-word N = 5 (the row and column of each value cost a division
-  // there), 2% slower for double-word N = 3 and 7 and, through a register
-  // increase that halves the resident CTAs, 23% slower for float32 N = 15
-  // (the compiler raises the register count at every N1 >= 11 of the float32
-  // kernels with it).
-  // (a gathered X, X[m] = u[gid[m]], is read one row per thread)
-  constexpr bool kRowsCoalesced =
-      XS::kDirect && ((sizeof(typename P::IO) == 4 && (N1 == 2 || N1 == 4 || N1 == 8)) || (P::kRoll && N1 == 16));
+  // pass 0: the elements into padded shared memory, each thread its own
+  // t-fiber: for every k a warp reads consecutive (i, j), so the loads are
+  // coalesced, and the shared-memory addresses need no division.  Against one
+  // i-row per thread (64 contiguous bytes per lane at N1 = 8) this matters most
+  // where a call is a fraction of a wave: order 7, 512 elements in double-word
+  // pairs 14.3 -> 12.3 us.  In native arithmetic D_t x starts from the
+  // registers that were just loaded.
   // Policies with kScaleIO (float64 data in float32 pairs): X is converted
-  // directly, and the threads test whether a row's largest magnitude lies
-  // outside the direct range (row_direct).  If any row of the block does, the
+  // directly, and the threads test whether their fiber's largest magnitude lies
+  // outside the direct range (row_direct).  If any fiber of the block does, the
   // block reads X again: each element is scaled by the power of two that
   // brings its largest magnitude into [1, 2) before the conversion, and its Y
-  // is scaled back on the way out.  (As a second kernel over a list of such
-  // blocks this cost every call a launch, 4 us with an empty list: order 7,
-  // 512 elements 18.4 -> 14.3 us per call; 131072 elements unchanged.)
-  bool wide = false;  // a row of this thread lies outside the direct range
-  if (act) {
-    using IO = typename P::IO;
-    if constexpr (kRowsCoalesced) {
-      wide = load_rows<P, N1, Sh::P, Sh::threads>(X.p + e0 * n3, nel * n3, xs, tid);
-    } else {
-      for (int row = tid; row < nel * N1 * N1; row += Sh::threads) {
-        const int64_t src = e0 * n3 + (int64_t)row * N1;
-        S *dst = xs + row * Sh::P;
-        int hmax = 0;       // the row's largest magnitude (upper 32 bits)
-        bool tiny = false;  // a nonzero value below from_io_direct's range
+  // is scaled back on the way out.
+  S *const x_e = xs + z * ES, *const r_e = b0 + z * ES, *const s_e = b1 + z * ES;
+  const int fr = Sh::at(0, qa, qb), fs = Sh::at(qa, 0, qb), ft = Sh::at(qa, jt, 0);
+  constexpr int str_r = 1, str_s = Sh::P, str_t = Sh::PK;
+  const int64_t own = e * n3 + qa + N1 * jt;  // node (qa, jt, 0); k: + k F
+  constexpr bool kRegX = !P::kRoll;  // native arithmetic: the fiber's x stays in registers for D_t x
+  V xt[kRegX ? N1 : 1];
+  bool wide = false;  // this thread's fiber (or row) lies outside the direct range
+  constexpr bool kRows = kRowLoads<P, N1>;
+  if constexpr (kRows) {
+    static_assert(ES == N1 * N1 * Sh::P, "value m of the block at (m / N1) P + m % N1");
+    for (int row = tid; row < nel * N1 * N1; row += Sh::threads) {
+      const int64_t src = e0 * n3 + (int64_t)row * N1;
+      S *dst = xs + row * Sh::P;
+      int hmax = 0;
+      bool tiny = false;
 #pragma unroll
-        for (int i = 0; i < N1; ++i) {
-          const IO v = X[src + i];
-          if constexpr (P::kScaleIO) {
-            hmax = max(hmax, mag_hi(v));
-            tiny |= dw::tiny_nonzero((unsigned)mag_hi(v));
-          }
-          dst[i] = P::st(P::from_io_direct(v));
-        }
-        if constexpr (P::kScaleIO) wide |= tiny || !row_direct(hmax);
+      for (int i = 0; i < N1; ++i) {
+        const typename P::IO v = X[src + i];
+        hmax = max(hmax, mag_hi(v));
+        tiny |= dw::tiny_nonzero((unsigned)mag_hi(v));
+        dst[i] = P::st(P::from_io_direct(v));
       }
+      wide |= tiny || !row_direct(hmax);
     }
-    if constexpr (GW > 0) {
+  } else if (live) {
+    using IO = typename P::IO;
+    int hmax = 0;       // the fiber's largest magnitude (upper 32 bits)
+    bool tiny = false;  // a nonzero value below from_io_direct's range
+#pragma unroll
+    for (int k = 0; k < N1; ++k) {
+      const IO v = X[own + k * F];
+      if constexpr (P::kScaleIO) {
+        hmax = max(hmax, mag_hi(v));
+        tiny |= dw::tiny_nonzero((unsigned)mag_hi(v));
+      }
+      const V xv = P::from_io_direct(v);
+      x_e[ft + k * str_t] = P::st(xv);
+      if constexpr (kRegX) xt[k] = xv;
+    }
+    if constexpr (P::kScaleIO) wide = tiny || !row_direct(hmax);
+  } else if constexpr (kRegX) {
+#pragma unroll
+    for (int k = 0; k < N1; ++k) xt[k] = P::lit(0.0);
+  }
+  if constexpr (GW > 0) {
+    if (act) {
       for (int m = tid; m < nel * GW; m += Sh::threads) sm.sgeo[(m / GW) * Buf::GWD + m % GW] = geo[e0 * GW + m];
     }
   }
@@ -733,19 +881,18 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     if (any_wide) {
       if (tid < EPB) sexp[tid] = 0;
       __syncthreads();
-      const int64_t srow = e * n3 + q * N1;  // row q of element z
       if (live) {
         int mx = 0;
 #pragma unroll 1
-        for (int i = 0; i < N1; ++i) mx = max(mx, exp_field(X[srow + i]));
+        for (int k = 0; k < N1; ++k) mx = max(mx, exp_field(X[kRows ? e * n3 + q * N1 + k : own + k * F]));
         atomicMax(&sexp[z], mx);
       }
       __syncthreads();
       if (live) {
         const typename P::IO sc = pow2i(io_shift(sexp[z]));
-        S *dst = xs + (z * N1 * N1 + q) * Sh::P;
 #pragma unroll 1
-        for (int i = 0; i < N1; ++i) dst[i] = P::st(P::from_io(X[srow + i] * sc));
+        for (int k = 0; k < N1; ++k)
+          x_e[kRows ? fr + k : ft + k * str_t] = P::st(P::from_io(X[kRows ? e * n3 + q * N1 + k : own + k * F] * sc));
       }
       __syncthreads();
     }
@@ -758,7 +905,6 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     if (live && q < 2 * N1) Geometry<P, N1, KIND>::axis_terms(sgeo_z, cx, q / N1, q % N1, sax_z + q * AXW);
   }
 
-  S *x_e = xs + z * ES, *r_e = b0 + z * ES, *s_e = b1 + z * ES;
   // Six fiber products in two rolled phase loops (one code copy of the fiber
   // product per matrix, D or D^T, so the constants stay immediate operands
   // and the instruction footprint fits the instruction cache):
@@ -768,8 +914,6 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   //   ph 3: t-fiber   D^T t -> registers (Y_t)
   //   ph 4: r-fibers  D^T r -> B0 (Y_r)  ph 5: s-fibers  D^T s -> B1 (Y_s)
   //   then the t-fiber owner stores Y = Y_t + Y_r + Y_s to HBM
-  const int fr = Sh::at(0, qa, qb), fs = Sh::at(qa, 0, qb), ft = Sh::at(qa, qb, 0);
-  constexpr int str_r = 1, str_s = Sh::P, str_t = Sh::P * N1;
   auto forward = [&](int ph) {
     if (ph == 2) __syncthreads();  // every r/s-fiber read of x is done before x is overwritten
     S *dst = ph == 0 ? r_e : (ph == 1 ? s_e : x_e);
@@ -787,8 +931,8 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     for (int ph = 0; ph < 3; ++ph) forward(ph);
   __syncthreads();
   {
-    // thread (i, j) = (qa, qb): geometry and G x along its own t-fiber
-    const int i = qa, j = qb;
+    // thread (i, j) = (qa, jt): geometry and G x along its own t-fiber
+    const int i = qa, j = jt;
     Geometry<P, N1, KIND> gm;
     gm.template prologue<AXS>(sgeo_z, cx, cw, i, j, (KIND == AX_GEOM_STORED && live) ? geo + e * 7 * n3 : nullptr,
                               (KIND == AX_GEOM_TRILINEAR_PARTIAL && live) ? lam + e * n3 : nullptr, sax_z);
@@ -835,7 +979,7 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     }
     __syncthreads();  // every Y_r, Y_s value is in B0, B1
     if (live) {
-      typename P::IO *ye = Y + e * n3 + qa + N1 * qb;
+      typename P::IO *ye = Y + own;
       auto yt_of = [&](int k) { return kYtRegs ? yt[kYtRegs ? k : 0] : P::ld(x_e + ft + k * str_t); };
       if (!sexp[EPB]) {
 #pragma unroll
@@ -863,34 +1007,56 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     // i, j: coalesced).  (IDLE threads skip every step but the barriers.)
     V tf[N1];
     if (act) {
-      forward(0);
+      contract_p<P, N1, KIND>(eoD, eo2D, xt, tf);
+      if constexpr (Sh::L::vec > 1) {
+        V fin_[N1], fout[N1];
+        load_row<N1, Sh::L::vec>(x_e + fr, fin_);
+        contract_p<P, N1, KIND>(eoD, eo2D, fin_, fout);
+        store_row<N1, Sh::L::vec>(r_e + fr, fout);
+      } else {
+        forward(0);
+      }
       forward(1);
-      V fin_[N1];
-#pragma unroll
-      for (int n = 0; n < N1; ++n) fin_[n] = P::ld(x_e + ft + n * str_t);
-      contract_p<P, N1, KIND>(eoD, eo2D, fin_, tf);
     }
     __syncthreads();  // every r/s fiber product is in B0, B1
     V yt[N1];
     if (act) {
-      const int i = qa, j = qb;
+      const int i = qa, j = jt;
       Geometry<P, N1, KIND> gm;
       const int64_t eg = live ? e : e0;
       gm.template prologue<AXS>(sgeo_z, cx, cw, i, j, KIND == AX_GEOM_STORED ? geo + eg * 7 * n3 : nullptr,
                                 KIND == AX_GEOM_TRILINEAR_PARTIAL ? lam + eg * n3 : nullptr, sax_z);
-#pragma unroll
-      for (int k = 0; k < N1; ++k) {
+      // (threads beyond the last element work on the block's first one's
+      // geometry: no branch per node, their results are not stored)
+      auto node = [&](int k) {
         const int sidx = ft + k * str_t;
         const V xv[3] = {P::ld(r_e + sidx), P::ld(s_e + sidx), tf[k]};
         V o3[3];
-        if (live) {
-          gm.apply(i + j * N1 + k * N1 * N1, P::cst(cx + k), P::cst(cw + k), xv, o3);
-        } else {
-          o3[0] = o3[1] = o3[2] = P::lit(0.0);
-        }
+        gm.apply(i + j * N1 + k * N1 * N1, P::cst(cx + k), P::cst(cw + k), xv, o3);
         r_e[sidx] = P::st(o3[0]);
         s_e[sidx] = P::st(o3[1]);
         tf[k] = o3[2];
+      };
+      if constexpr (kPackedGeo<P, N1, KIND>) {
+        const Geometry2<N1, KIND> g2(gm);
+#pragma unroll
+        for (int k = 0; k < N1 / 2; ++k) {
+          const int k2 = N1 - 1 - k, s1 = ft + k * str_t, s2 = ft + k2 * str_t;
+          const float2 xv[3] = {make_float2(r_e[s1], r_e[s2]), make_float2(s_e[s1], s_e[s2]),
+                                make_float2(tf[k], tf[k2])};
+          float2 o3[3];
+          g2.apply(i + j * N1 + k * N1 * N1, i + j * N1 + k2 * N1 * N1, make_float2(cx[k], cx[k2]), cw[k], xv, o3);
+          r_e[s1] = o3[0].x;
+          r_e[s2] = o3[0].y;
+          s_e[s1] = o3[1].x;
+          s_e[s2] = o3[1].y;
+          tf[k] = o3[2].x;
+          tf[k2] = o3[2].y;
+        }
+        if constexpr (N1 & 1) node(N1 / 2);
+      } else {
+#pragma unroll
+        for (int k = 0; k < N1; ++k) node(k);
       }
       contract_p<P, N1, KIND>(eoDT, eo2DT, tf, yt);
     }
@@ -901,6 +1067,14 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
       S *buf = d == 0 ? r_e : s_e;
       const int base = d == 0 ? fr : fs, stride = d == 0 ? str_r : str_s;
       V fin_[N1], fout[N1];
+      if constexpr (Sh::L::vec > 1) {
+        if (d == 0) {
+          load_row<N1, Sh::L::vec>(buf + base, fin_);
+          contract_p<P, N1, KIND>(eoDT, eo2DT, fin_, fout);
+          store_row<N1, Sh::L::vec>(buf + base, fout);
+          continue;
+        }
+      }
 #pragma unroll
       for (int n = 0; n < N1; ++n) fin_[n] = P::ld(buf + base + n * stride);
       contract_p<P, N1, KIND>(eoDT, eo2DT, fin_, fout);
@@ -909,7 +1083,7 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     }
     __syncthreads();  // every Y_r, Y_s value is in B0, B1
     if (live) {
-      typename P::IO *ye = Y + e * n3 + qa + N1 * qb;
+      typename P::IO *ye = Y + own;
 #pragma unroll
       for (int k = 0; k < N1; ++k) {
         const int sidx = ft + k * str_t;
@@ -990,7 +1164,7 @@ __global__ void __launch_bounds__(Shape<N1, 1, kEpb<P, N1, KIND>>::threads)
 // Dynamic shared memory of a kernel of this shape.
 template <class P, int N1, int KIND, int EM>
 size_t launch_smem(const void *kernel) {
-  using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
+  using Sh = Shape<N1, EM, kEpb<P, N1, KIND>, kLayout<P, N1, KIND>>;
   const size_t smem = (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S);
   if constexpr (P::kTargetWarpsPerSM > 0 && N1 == 8 &&
                 (KIND == AX_GEOM_TRILINEAR || KIND == AX_GEOM_TRILINEAR_PARTIAL)) {
