@@ -178,8 +178,11 @@ ax_status ax_diag(ax_ctx *c, void *diag_local, void *stream);
  *   so it has its own entry point, pcg_solve_learned(ctx, mlp, ...).
  *   Other values return AX_EUNSUPPORTED.  Stops when ||r||_2 <= rtol ||b||_2 or after maxit iterations
  *   (AX_ENOTCONV).  *iters and *relres (host) report the outcome.
- * One iteration is four kernels (direction + scatter, AxLocal, gather + p.w
- * with alpha, update + r.z, r.r with the convergence test and beta); every
+ * One iteration is two kernels for AX_FP32 and AX_F64DW contexts whose every
+ * global node belongs to an element (AxLocal with the direction, the update of
+ * x and alpha fused in; gather + update + r.z, r.r with the convergence test
+ * and beta), else four (direction + scatter, AxLocal, gather + p.w with alpha,
+ * update and test); every
  * scalar stays on the device and the grid-level sums are finished in the
  * producing kernel in a fixed order (deterministic).  Blocks of 16
  * iterations run as one CUDA graph on a private stream, ordered after and

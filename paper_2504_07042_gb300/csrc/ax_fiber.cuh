@@ -29,6 +29,7 @@
 #include "ax_internal.h"
 #include "dw.cuh"
 #include "dw2.cuh"
+#include "reduce.cuh"
 #include "tables.cuh"
 
 namespace ax {
@@ -733,19 +734,63 @@ struct GeoWords {
   static constexpr int value = (KIND == AX_GEOM_STORED) ? 0 : (KIND == AX_GEOM_PARALLELEPIPED ? kParWords : kVertexWords);
 };
 
-// Sources of X: in place (element e's values at X[e n3 + m]), or the local
-// copies of a global vector, X[m] = u[gid[m]] (the scatter Q u of Eq. 1,
-// fused into the load).
+// Sources of X: in place (element e's values at X[e n3 + m]), or formed from
+// the assembled vectors of a CG iteration (XCg).
 template <typename IO>
 struct XDirect {
+  static constexpr bool kCg = false;
   const IO *__restrict__ p;
   __device__ __forceinline__ IO operator[](int64_t m) const { return p[m]; }
 };
+// The local copies of a global vector, X[m] = u[gid[m]].
 template <typename IO>
 struct XGather {
+  static constexpr bool kCg = false;
   const IO *__restrict__ u;
   const gidx *__restrict__ gid;
   __device__ __forceinline__ IO operator[](int64_t m) const { return u[gid[m]]; }
+};
+
+// The search direction of a CG iteration, formed at each local copy while it
+// is loaded: p_new[g] = z[g] + beta p[g].  The thread that loads a node's
+// first copy also stores p_new and brings x up to date, x += alpha p, with
+// the last iteration's alpha and direction.  p_new goes to another vector
+// than p, so every copy sees the same p.  Y is stored by rank (CgArgs).
+template <typename IO>
+struct XCg {
+  static constexpr bool kCg = true;
+  static constexpr int kBatch = 8;  // nodes whose loads are in flight together
+  const gidx *__restrict__ own;
+  const gidx *__restrict__ rank;
+  const IO *__restrict__ z;
+  const IO *__restrict__ p;
+  IO *pn, *x, *U;
+  IO alpha, beta;
+  // local copies m, m + step, ... (n of them; all loads before the first store)
+  template <int n>
+  __device__ __forceinline__ void get(int64_t m, int step, IO *out) const {
+    gidx g[n];
+    IO zv[n], pv[n], xv[n];
+#pragma unroll
+    for (int u = 0; u < n; ++u) g[u] = own[m + u * step];
+#pragma unroll
+    for (int u = 0; u < n; ++u) {
+      const gidx h = g[u] & 0x7fffffff;
+      zv[u] = z[h];
+      pv[u] = p[h];
+      xv[u] = g[u] < 0 ? x[h] : IO(0);
+    }
+#pragma unroll
+    for (int u = 0; u < n; ++u) {
+      const gidx h = g[u] & 0x7fffffff;
+      out[u] = zv[u] + beta * pv[u];
+      if (g[u] < 0) {
+        pn[h] = out[u];
+        x[h] = xv[u] + alpha * pv[u];
+      }
+    }
+  }
+  __device__ __forceinline__ IO operator[](int64_t m) const { return U[m]; }  // after the block's loads (float64 IO)
 };
 
 // Shared-memory buffers of one block of EPB elements.
@@ -786,8 +831,11 @@ struct FiberSmem {
 // threads than the order's shape (a CTA shaped for several orders); those
 // threads only take part in the barriers.
 // ---------------------------------------------------------------------------
+// Returns, with X the direction of a CG iteration (XCg), this thread's share
+// of X . Y (the dot product p . A p needs no assembled vector: p^T Q^T Y over
+// the local copies), else 0.
 template <class P, int N1, int KIND, int EM, bool IDLE, class XS, int EPB0 = kEpb<P, N1, KIND>>
-__device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB0> &sm, const int tid, const int64_t e0,
+__device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIND, EM, EPB0> &sm, const int tid, const int64_t e0,
                                             const int nel, const typename P::S *__restrict__ geo,
                                             const typename P::S *__restrict__ lam, const XS &X,
                                             typename P::IO *__restrict__ Y) {
@@ -817,6 +865,7 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   S *const sax_z = sm.sax + (act && AXS ? z : 0) * Buf::AXD;
   const int64_t e = e0 + z;
   const bool live = act && z < nel;
+  typename P::IO xy = 0;
 
   // pass 0: the elements into padded shared memory, each thread its own
   // t-fiber: for every k a warp reads consecutive (i, j), so the loads are
@@ -838,7 +887,7 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
   constexpr bool kRegX = !P::kRoll;  // native arithmetic: the fiber's x stays in registers for D_t x
   V xt[kRegX ? N1 : 1];
   bool wide = false;  // this thread's fiber (or row) lies outside the direct range
-  constexpr bool kRows = kRowLoads<P, N1>;
+  constexpr bool kRows = kRowLoads<P, N1> && !XS::kCg;
   if constexpr (kRows) {
     static_assert(ES == N1 * N1 * Sh::P, "value m of the block at (m / N1) P + m % N1");
     for (int row = tid; row < nel * N1 * N1; row += Sh::threads) {
@@ -859,9 +908,23 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     using IO = typename P::IO;
     int hmax = 0;       // the fiber's largest magnitude (upper 32 bits)
     bool tiny = false;  // a nonzero value below from_io_direct's range
+    IO cgv[8];
 #pragma unroll
     for (int k = 0; k < N1; ++k) {
-      const IO v = X[own + k * F];
+      IO v;
+      if constexpr (XS::kCg) {
+        constexpr int B = XS::kBatch, R = N1 % B ? N1 % B : B;
+        if (k % B == 0) {
+          if (k + B <= N1)
+            X.template get<B>(own + k * F, F, cgv);
+          else
+            X.template get<R>(own + k * F, F, cgv);
+        }
+        v = cgv[k % B];
+        if constexpr (P::kScaleIO) X.U[own + k * F] = v;  // read back for the dot product and the scaled reload
+      } else {
+        v = X[own + k * F];
+      }
       if constexpr (P::kScaleIO) {
         hmax = max(hmax, mag_hi(v));
         tiny |= dw::tiny_nonzero((unsigned)mag_hi(v));
@@ -984,22 +1047,43 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     }
     __syncthreads();  // every Y_r, Y_s value is in B0, B1
     if (live) {
-      typename P::IO *ye = Y + own;
       auto yt_of = [&](int k) { return kYtRegs ? yt[kYtRegs ? k : 0] : P::ld(x_e + ft + k * str_t); };
-      if (!sexp[EPB]) {
+      auto store = [&](auto y_of) {
+        if constexpr (XS::kCg) {
+          constexpr int B = 4;  // places and x of B nodes are loaded before the first of them is stored
 #pragma unroll
-        for (int k = 0; k < N1; ++k) {
-          const int sidx = ft + k * str_t;
-          ye[k * N1 * N1] = P::sum3_io_direct(yt_of(k), P::ld(r_e + sidx), P::ld(s_e + sidx));
+          for (int k0 = 0; k0 < N1; k0 += B) {
+            gidx at[B];
+            typename P::IO xv[B];
+#pragma unroll
+            for (int k = k0; k < N1 && k < k0 + B; ++k) {
+              at[k - k0] = X.rank[own + k * F];
+              xv[k - k0] = X[own + k * F];
+            }
+#pragma unroll
+            for (int k = k0; k < N1 && k < k0 + B; ++k) {
+              const typename P::IO y = y_of(k);
+              Y[at[k - k0]] = y;
+              xy += xv[k - k0] * y;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < N1; ++k) Y[own + k * F] = y_of(k);
         }
+      };
+      if (!sexp[EPB]) {
+        store([&](int k) {
+          const int sidx = ft + k * str_t;
+          return P::sum3_io_direct(yt_of(k), P::ld(r_e + sidx), P::ld(s_e + sidx));
+        });
       } else {
         // the element entered as X 2^d: undo it (exact)
         const typename P::IO ysc = pow2i(-io_shift(sexp[z]));
-#pragma unroll
-        for (int k = 0; k < N1; ++k) {
+        store([&](int k) {
           const int sidx = ft + k * str_t;
-          ye[k * N1 * N1] = P::sum3_io(yt_of(k), P::ld(r_e + sidx), P::ld(s_e + sidx)) * ysc;
-        }
+          return P::sum3_io(yt_of(k), P::ld(r_e + sidx), P::ld(s_e + sidx)) * ysc;
+        });
       }
     }
   } else {
@@ -1088,16 +1172,27 @@ __device__ __forceinline__ void fiber_block(const FiberSmem<P, N1, KIND, EM, EPB
     }
     __syncthreads();  // every Y_r, Y_s value is in B0, B1
     if (live) {
-      typename P::IO *ye = Y + own;
+      gidx at[XS::kCg ? N1 : 1];
+      if constexpr (XS::kCg) {
+#pragma unroll
+        for (int k = 0; k < N1; ++k) at[k] = X.rank[own + k * F];
+      }
 #pragma unroll
       for (int k = 0; k < N1; ++k) {
         const int sidx = ft + k * str_t;
-        ye[k * N1 * N1] = P::sum3_io(yt[k], P::ld(r_e + sidx), P::ld(s_e + sidx));
+        const V y = P::sum3_io(yt[k], P::ld(r_e + sidx), P::ld(s_e + sidx));
+        if constexpr (XS::kCg) {
+          Y[at[k]] = y;
+          xy += P::ld(x_e + sidx) * y;  // X still lies where it was loaded
+        } else {
+          Y[own + k * F] = y;
+        }
       }
     }
   }
 
   __syncthreads();  // the next block reuses the shared buffers
+  return xy;
 }
 
 // ---------------------------------------------------------------------------
@@ -1127,6 +1222,75 @@ __global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads, kMi
     const int64_t e0 = blk * EPB;
     const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
     fiber_block<P, N1, KIND, EM, false>(sm, tid, e0, nel, geo, lam, XDirect<typename P::IO>{X}, Y);
+  }
+}
+
+// The policies with a CG form of the kernel: those that solvers run on by
+// default (native FP64 and the tensor-core kernels take the general iteration).
+template <class P>
+constexpr bool kHasCg = P::kRoll || sizeof(typename P::IO) == 4;
+
+// First half of a CG iteration (ax_gs.cu): p_new = z + beta p formed in the
+// loads, x += alpha p, W = A_e p_new, and alpha = r.z / p.w by the CTA that
+// arrives last.  It takes the place of a direction-and-scatter kernel, the
+// plain AxLocal and a dot product; the vectors' loads overlap the arithmetic
+// that bounds the operator: order 7, 4096 elements, double-word 78 us (AxLocal
+// alone 60), float32 20 (10); the kernels whose place it takes took 38 and 25.
+// (A resident CTA per slot that loops over the blocks keeps the CTAs' phases
+// in step: 86 us instead of 78.)
+template <class P, int N1, int KIND>
+__global__ void __launch_bounds__(Shape<N1, 1, kEpb<P, N1, KIND>>::threads, kMinCtas<P, N1, KIND>)
+    ax_fiber_cg_kernel(int64_t E, const typename P::S *__restrict__ geo, const typename P::S *__restrict__ lam,
+                       const CgArgs c, typename P::IO *__restrict__ Y) {
+  using Sh = Shape<N1, 1, kEpb<P, N1, KIND>>;
+  using Buf = FiberSmem<P, N1, KIND, 1>;
+  using S = typename P::S;
+  using IO = typename P::IO;
+  constexpr int EPB = Sh::EPB;
+  const double stop = c.S[6], alpha = c.S[10], beta = c.S[11];
+  if (stop != 0.0) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ S sgeo[EPB][Buf::GWD];
+  __shared__ S sax[Buf::AXS ? EPB : 1][Buf::AXD];
+  __shared__ int sexp[P::kScaleIO ? EPB + 1 : 1];
+  Buf sm;
+  sm.xs = (S *)smem_raw;
+  sm.sgeo = &sgeo[0][0];
+  sm.sax = &sax[0][0];
+  sm.sexp = sexp;
+  const int tid = threadIdx.x;
+  const XCg<IO> X{c.own, c.rank, (const IO *)c.z, (const IO *)c.p, (IO *)c.pn, (IO *)c.x, (IO *)c.U, (IO)alpha, (IO)beta};
+  const int64_t nblk = (E + EPB - 1) / EPB;
+  IO dot = 0;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    const int64_t e0 = blk * EPB;
+    const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
+    dot += fiber_block<P, N1, KIND, 1, false>(sm, tid, e0, nel, geo, lam, X, Y);
+  }
+  // sums in a fixed order: over the CTA's threads in the vectors' type, then
+  // over the CTAs in double (the shared buffers are free: fiber_block ends
+  // with a barrier); results in thread 0
+  auto sum_cta = [&](auto v) {
+    using T = decltype(v);
+    T *sums = (T *)smem_raw;
+    sums[tid] = v;
+    __syncthreads();
+    T s = 0;
+    if (tid < 32) {
+      for (int q = tid; q < Sh::threads; q += 32) s += sums[q];
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+    return s;
+  };
+  const IO mine = sum_cta(dot);
+  if (tid == 0) c.part[blockIdx.x] = (double)mine;
+  if (!red::arrive_last(c.cnt)) return;
+  double s = 0.0;
+  for (int q = tid; q < (int)gridDim.x; q += Sh::threads) s += __ldcg(c.part + q);
+  const double pw = sum_cta(s);
+  if (tid == 0) {
+    c.S[1] = pw;
+    c.S[10] = pw != 0.0 ? c.S[0] / pw : 0.0;
   }
 }
 
@@ -1214,6 +1378,29 @@ cudaError_t launch_ax_em(const AxArgs &a) {
   return cudaGetLastError();
 }
 
+// The CG form (a.cg); with E = 0 the kernel is only prepared (before a
+// capture).  A partial sum per CTA: at most E of them.
+template <class P, int N1, int KIND>
+cudaError_t launch_ax_cg(const AxArgs &a) {
+  using Sh = Shape<N1, 1, kEpb<P, N1, KIND>, kLayout<P, N1, KIND>>;
+  static_assert(Sh::threads >= 32 && (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S) >= Sh::threads * sizeof(double),
+                "a whole warp and a double per thread for the sums");
+  static const size_t smem = launch_smem<P, N1, KIND, 1>((const void *)ax_fiber_cg_kernel<P, N1, KIND>);
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(ax_fiber_cg_kernel<P, N1, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  const int64_t nblk = (a.E + Sh::EPB - 1) / Sh::EPB;
+  if (nblk <= 0) return cudaSuccess;
+  if (nblk > 0x7fffffffLL) return cudaErrorInvalidValue;
+  ax_fiber_cg_kernel<P, N1, KIND><<<(unsigned)nblk, Sh::threads, smem, a.stream>>>(
+      a.E, (const typename P::S *)a.geo, (const typename P::S *)a.lam, *a.cg, (typename P::IO *)a.Y);
+  return cudaGetLastError();
+}
+
 template <class P, int N1, int KIND>
 cudaError_t launch_fiber_n(const AxArgs &a, double *G_out) {
   using Sh = Shape<N1, 1, kEpb<P, N1, KIND>>;
@@ -1224,6 +1411,12 @@ cudaError_t launch_fiber_n(const AxArgs &a, double *G_out) {
     factors_fiber_kernel<P, N1, KIND><<<(unsigned)blocks, Sh::threads, 0, a.stream>>>(
         a.E, (const typename P::S *)a.geo, (const typename P::S *)a.lam, G_out);
     return cudaGetLastError();
+  }
+  if (a.cg) {
+    if constexpr (kHasCg<P>)
+      return launch_ax_cg<P, N1, KIND>(a);
+    else
+      return cudaErrorNotSupported;
   }
   if constexpr (P::kTiles > 1) {
     if (a.tile == 1) return launch_ax_em<P, N1, KIND, 2>(a);

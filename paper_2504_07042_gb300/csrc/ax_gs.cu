@@ -189,6 +189,23 @@ __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152)
   }
 }
 
+// the end of an iteration, by the last block: beta, the count, the test
+__device__ __forceinline__ void finish_iteration(double *S, double rz_new, double rr_new) {
+  S[4] = rz_new;
+  S[2] = rr_new;
+  S[11] = S[0] != 0.0 ? rz_new / S[0] : 0.0;
+  S[0] = rz_new;
+  const double it = S[9] + 1.0;
+  S[9] = it;
+  if (rr_new <= S[8]) {
+    S[6] = 1.0;
+    S[7] = it;
+  } else if (!(rr_new == rr_new)) {
+    S[6] = 1.0;
+    S[7] = -it;
+  }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152)
     update_check_kernel(int64_t n, double *__restrict__ S, const T *__restrict__ p, const T *__restrict__ w,
@@ -242,21 +259,102 @@ __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152)
   if (!red::arrive_last(cnt)) return;
   double rz_new, rr_new;
   red::sum_partials2(part_rz, part_rr, gridDim.x, rz_new, rr_new);
-  if (threadIdx.x == 0) {
-    S[4] = rz_new;
-    S[2] = rr_new;
-    S[11] = S[0] != 0.0 ? rz_new / S[0] : 0.0;
-    S[0] = rz_new;
-    const double it = S[9] + 1.0;
-    S[9] = it;
-    if (rr_new <= S[8]) {
-      S[6] = 1.0;
-      S[7] = it;
-    } else if (!(rr_new == rr_new)) {
-      S[6] = 1.0;
-      S[7] = -it;
+  if (threadIdx.x == 0) finish_iteration(S, rz_new, rr_new);
+}
+
+// ---------------------------------------------------------------------------
+// The fused iteration (FP32 and double-word contexts whose every global node
+// has a local copy): two launches instead of four.
+//   AxLocal in its CG form (ax_fiber_cg_kernel)
+//                      p_new = z + beta p and x += alpha_last p while X is
+//                      loaded; W = A_e Q p_new; alpha from p^T Q^T W, summed
+//                      over the local copies
+//   gather_update      r -= alpha Q^T W; z = M^-1 r; r.z, r.r; test; beta
+// Neither Q p nor w = Q^T W is written to memory, and x is one update behind,
+// brought up to date by finish_x.  Bound by HBM and L2 traffic and, in
+// float64, by the FP64 pipe (5 to 6 operations per node at 2 per clock and
+// SM).  Measured on GB300 per iteration at order 7, 4096 elements, against the
+// four launches of the general one: double-word 104 against 115 us (operator
+// 78, gather_update 27), float32 33 against 48 us (20 and 13).
+// ---------------------------------------------------------------------------
+// gather_update's blocks per SM and nodes per thread whose loads are in flight
+// together.  Double: two nodes in 40 registers, so that 48 warps per SM keep
+// the FP64 pipe busy while others wait for loads (four nodes in 64 registers
+// and 32 warps: 37 against 30 us for 1.44e6 nodes; 64 warps spill).  Float, whose
+// arithmetic is cheap: four (two nodes and 64 warps: 13.6 against 13.3 us).
+template <typename T>
+struct Fuse {
+  static constexpr int kPerSm = sizeof(T) == 8 ? 6 : 4, kU = sizeof(T) == 8 ? 2 : 4;
+  static constexpr int kBlocks = 152 * kPerSm;
+};
+constexpr int kPartials = 152 * 6;  // doubles per array of block sums (>= kRedBlocks, Fuse::kBlocks)
+// Blocks for n nodes: one wave at most, and no fewer than 256 nodes each (small
+// systems are bound by the launch and by the sum over the blocks' partials).
+template <typename T>
+inline int fused_blocks(int64_t n) {
+  const int64_t b = (n + kRedThreads - 1) / kRedThreads;
+  return (int)(b < 1 ? 1 : (b < Fuse<T>::kBlocks ? b : Fuse<T>::kBlocks));
+}
+// r -= alpha Q^T Y, z = M^-1 r, the sums, the test and beta.  The operator left
+// every node's copies side by side, at the CSR's own offsets: one coalesced
+// load away, with no index to fetch first (copies gathered through the index
+// list: 42 us in double and 18.6 in float for 1.44e6 nodes; now 27.4 and 13.3).
+// Blocks take groups of 256 nodes in turn: a block with a contiguous share can
+// get whole planes of nodes with two to eight copies (30 us in double).
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads, Fuse<T>::kPerSm)
+    gather_update_kernel(int64_t n, const gidx *__restrict__ off, const T *__restrict__ Y, T *__restrict__ r,
+                         T *__restrict__ z, const T *__restrict__ inv, const uint8_t *__restrict__ mask,
+                         double *__restrict__ part_rz, double *__restrict__ part_rr, unsigned *__restrict__ cnt,
+                         double *__restrict__ S) {
+  constexpr int U = Fuse<T>::kU;
+  if (S[6] != 0.0) return;
+  const T alpha = (T)S[10];
+  T rz = T(0), rr = T(0);
+  // 256 nodes in turn to every block, U such groups at a time
+  const int64_t step = (int64_t)gridDim.x * kRedThreads;
+  for (int64_t base = (int64_t)blockIdx.x * kRedThreads; base < n; base += U * step) {
+    T s[U], rv[U], iv[U];
+    gidx b[U], c[U];
+    bool mv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t g = base + threadIdx.x + u * step;
+      const bool on = g < n;
+      b[u] = on ? off[g] : 0;
+      c[u] = on ? off[g + 1] - b[u] : 0;
+      rv[u] = on ? r[g] : T(0);
+      iv[u] = on && inv ? inv[g] : T(1);
+      mv[u] = !on || (mask && mask[g]);
+    }
+    red::gather_copies<T, U>(Y, b, c, s);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t g = base + threadIdx.x + u * step;
+      if (g >= n) break;
+      if (mv[u]) s[u] = T(0);
+      const T rg = rv[u] - alpha * s[u];
+      T zg = inv ? rg * iv[u] : rg;
+      if (mv[u]) zg = T(0);
+      r[g] = rg;
+      z[g] = zg;
+      rz += rg * zg;
+      rr += rg * rg;
     }
   }
+  red::block_reduce2_store<T>(rz, rr, part_rz + blockIdx.x, part_rr + blockIdx.x);
+  if (!red::arrive_last(cnt)) return;
+  double rz_new, rr_new;
+  red::sum_partials2(part_rz, part_rr, gridDim.x, rz_new, rr_new);
+  if (threadIdx.x == 0) finish_iteration(S, rz_new, rr_new);
+}
+
+// x += alpha p: the update that the fused iteration still owes after its last one
+template <typename T>
+__global__ void finish_x_kernel(int64_t n, const double *__restrict__ S, const T *__restrict__ p, T *__restrict__ x) {
+  const T alpha = (T)S[10];
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x)
+    x[g] += alpha * p[g];
 }
 
 __global__ void set_kernel(double *S, int idx, double v) { S[idx] = v; }
@@ -299,6 +397,17 @@ __global__ void invert_kernel(int64_t n, const T *__restrict__ d, T *__restrict_
     inv[g] = (mask && mask[g]) ? T(0) : T(1) / d[g];
 }
 
+// own and rank of a plan (GsPlan) from its CSR map
+__global__ void own_rank_kernel(int64_t n_local, const gidx *__restrict__ off, const gidx *__restrict__ idx,
+                                const gidx *__restrict__ gid, gidx *__restrict__ own, gidx *__restrict__ rank) {
+  constexpr gidx kFlag = INT32_MIN;  // the sign bit: indices stay below 2^31
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n_local; q += (int64_t)gridDim.x * blockDim.x) {
+    const gidx m = idx[q], g = gid[m];
+    rank[m] = (gidx)q;
+    own[m] = off[g] == q ? g | kFlag : g;
+  }
+}
+
 inline unsigned grid_for(int64_t n, int block = 256) {
   int64_t g = (n + block - 1) / block;
   if (g < 1) g = 1;
@@ -329,11 +438,16 @@ cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int6
     ++off[g + 1];
   }
   if (*bad_ids) return cudaSuccess;
-  for (int64_t g = 0; g < n_global; ++g) off[g + 1] += off[g];
+  plan.complete = n_global > 0;
+  for (int64_t g = 0; g < n_global; ++g) {
+    plan.complete &= off[g + 1] != 0;
+    off[g + 1] += off[g];
+  }
   std::vector<gidx> idx((size_t)n_local), gid32((size_t)n_local), fill(off.begin(), off.end() - 1);
   for (int64_t m = 0; m < n_local; ++m) {
-    gid32[m] = (gidx)gid[m];
-    idx[fill[gid[m]]++] = (gidx)m;  // increasing local order per global node
+    const int64_t g = gid[m];
+    gid32[m] = (gidx)g;
+    idx[fill[g]++] = (gidx)m;  // increasing local order per global node
   }
   plan.n_global = n_global;
   plan.n_local = n_local;
@@ -354,10 +468,25 @@ cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int6
   return e;
 }
 
+bool gs_fused_view(const GsPlan &plan, cudaStream_t s) {
+  if (!plan.complete) return false;
+  if (plan.own) return true;
+  if (cudaMalloc(&plan.own, sizeof(gidx) * 2 * plan.n_local) != cudaSuccess) {
+    cudaGetLastError();  // no room for it: the general iteration
+    plan.own = nullptr;
+    return false;
+  }
+  plan.rank = plan.own + plan.n_local;
+  gs::own_rank_kernel<<<gs::grid_for(plan.n_local), 256, 0, s>>>(plan.n_local, plan.off, plan.idx, plan.gid, plan.own,
+                                                                 plan.rank);
+  return true;
+}
+
 void gs_free(GsPlan &plan) {
   cudaFree(plan.off);
   cudaFree(plan.idx);
   cudaFree(plan.gid);
+  cudaFree(plan.own);  // and rank
   cudaFree(plan.mask);
   plan = GsPlan();
 }
@@ -395,24 +524,26 @@ cudaError_t gs_scatter_run(const GsPlan &p, bool f64, const void *u, void *U, cu
 // Work vectors of one CG solve (allocated once per solve, reused across the
 // inner solves of the mixed-precision driver), with the private stream and
 // the instantiated graph of kCheck iterations.
-constexpr int kCheck = 16;  // iterations per graph launch (between host checks)
+constexpr int kCheck = 16;  // iterations per graph launch (between host checks); even (fused_iteration's parity)
 
 template <typename T>
 struct PcgWork {
   int64_t n = 0, nl = 0;
   T *r = nullptr, *z = nullptr, *p = nullptr, *w = nullptr, *Ul = nullptr, *Yl = nullptr, *inv = nullptr;
   double *S = nullptr, *part = nullptr, *hS = nullptr;
+  double *part_ax = nullptr;  // fused iteration: a partial sum per AxLocal CTA (at most one per element)
   unsigned *cnt = nullptr;
   cudaStream_t cs = nullptr;
   cudaEvent_t ev = nullptr;
   cudaGraphExec_t exec = nullptr;
-  const void *graph_b = nullptr;  // the (b, x, preconditioner, operator) the graph was captured for
+  const void *graph_b = nullptr;  // the (b, x, preconditioner, operator, form) the graph was captured for
   void *graph_x = nullptr;
   bool graph_jac = false;
   const void *graph_op = nullptr;
+  bool graph_fused = false;
   bool jac = false;  // Jacobi on: inv holds the inverted diagonal
   T *inv_or_null() const { return jac ? inv : nullptr; }
-  cudaError_t alloc(int64_t n_, int64_t nl_, bool jacobi) {
+  cudaError_t alloc(int64_t n_, int64_t nl_, int64_t E) {
     n = n_;
     nl = nl_;
     cudaError_t e = cudaMalloc(&r, sizeof(T) * n);
@@ -421,11 +552,11 @@ struct PcgWork {
     if (e == cudaSuccess) e = cudaMalloc(&w, sizeof(T) * n);
     if (e == cudaSuccess) e = cudaMalloc(&Ul, sizeof(T) * nl);
     if (e == cudaSuccess) e = cudaMalloc(&Yl, sizeof(T) * nl);
-    (void)jacobi;
+    if (e == cudaSuccess) e = cudaMalloc(&part_ax, sizeof(double) * (E > 0 ? E : 1));
     if (e == cudaSuccess) e = cudaMalloc(&inv, sizeof(T) * n);
     if (e == cudaSuccess) e = cudaMalloc(&S, sizeof(double) * gs::kScalars);
     if (e == cudaSuccess) e = cudaMemset(S, 0, sizeof(double) * gs::kScalars);
-    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * 3 * gs::kRedBlocks);
+    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * 3 * gs::kPartials);
     if (e == cudaSuccess) e = cudaMalloc(&cnt, sizeof(unsigned) * 2);
     if (e == cudaSuccess) e = cudaMemset(cnt, 0, sizeof(unsigned) * 2);
     if (e == cudaSuccess) e = cudaMallocHost(&hS, sizeof(double) * gs::kScalars);
@@ -438,7 +569,7 @@ struct PcgWork {
     if (ev) cudaEventDestroy(ev);
     if (cs) cudaStreamDestroy(cs);
     cudaFree(r); cudaFree(z); cudaFree(p); cudaFree(w); cudaFree(Ul); cudaFree(Yl); cudaFree(inv);
-    cudaFree(S); cudaFree(part); cudaFree(cnt); cudaFreeHost(hS);
+    cudaFree(S); cudaFree(part); cudaFree(part_ax); cudaFree(cnt); cudaFreeHost(hS);
     *this = PcgWork();
   }
 };
@@ -456,6 +587,39 @@ static cudaError_t pcg_iteration(const GsPlan &P, const AxArgs &a, cudaError_t (
                                                    W.S);
   gs::update_check_kernel<T><<<RB, RT, 0, s>>>(n, W.S, W.p, W.w, x, W.r, W.z, W.inv_or_null(), P.mask, W.part, W.part + RB,
                                                W.cnt + 1);
+  return cudaGetLastError();
+}
+
+// Whether the fused iteration applies: the launcher has a CG form and every
+// global node has a local copy to own it (a node without one is touched by
+// the general iteration's vector kernels only).
+static bool fused_ok(const GsPlan &P, cudaError_t (*launch)(const AxArgs &), cudaStream_t s) {
+  return (launch == launch_ax_fp32 || launch == launch_ax_dw) && gs_fused_view(P, s);
+}
+
+// One fused CG iteration (two launches) on stream s; k: its number since the
+// solve began (only its parity counts: p and w take turns as the direction).
+template <typename T>
+static cudaError_t fused_iteration(const GsPlan &P, AxArgs a, cudaError_t (*launch)(const AxArgs &), PcgWork<T> &W,
+                                   T *x, int k, cudaStream_t s) {
+  const int RB = gs::fused_blocks<T>(P.n_global);
+  CgArgs c;
+  c.own = P.own;
+  c.rank = P.rank;
+  c.z = W.z;
+  c.p = (k & 1) ? W.w : W.p;
+  c.pn = (k & 1) ? W.p : W.w;
+  c.x = x;
+  c.U = W.Ul;
+  c.S = W.S;
+  c.part = W.part_ax;
+  c.cnt = W.cnt;
+  a.cg = &c;
+  a.stream = s;
+  const cudaError_t e = launch(a);
+  if (e != cudaSuccess) return e;
+  gs::gather_update_kernel<T><<<RB, gs::kRedThreads, 0, s>>>(P.n_global, P.off, W.Yl, W.r, W.z, W.inv_or_null(),
+                                                             P.mask, W.part, W.part + gs::kPartials, W.cnt + 1, W.S);
   return cudaGetLastError();
 }
 
@@ -501,18 +665,31 @@ static cudaError_t pcg_core(const GsPlan &P, const AxArgs &base, cudaError_t (*l
     gs::set_kernel<<<1, 1, 0, s>>>(S, 6, 0.0);
     gs::set_kernel<<<1, 1, 0, s>>>(S, 9, 0.0);
     gs::set_kernel<<<1, 1, 0, s>>>(S, 11, 0.0);  // first direction: p = z
+    gs::set_kernel<<<1, 1, 0, s>>>(S, 10, 0.0);  // fused: no update of x owed yet
     cudaStream_t cs = W.cs;
-    e = cudaEventRecord(W.ev, s);
+    const bool fused = fused_ok(P, launch, s);
+    auto iteration = [&](int k) {
+      return fused ? fused_iteration<T>(P, a, launch, W, x, k, cs) : pcg_iteration<T>(P, a, launch, W, x, cs);
+    };
+    if (fused) {
+      // the kernel is loaded and its shared memory set before the capture
+      AxArgs none = a;
+      const CgArgs c;
+      none.E = 0;
+      none.cg = &c;
+      e = launch(none);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(W.ev, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, W.ev, 0);
     a.stream = cs;
     if (e == cudaSuccess && maxit >= kCheck &&
         (!W.exec || W.graph_b != (const void *)b || W.graph_x != (void *)x || W.graph_jac != W.jac ||
-         W.graph_op != base.geo)) {
+         W.graph_op != base.geo || W.graph_fused != fused)) {
       if (W.exec) cudaGraphExecDestroy(W.exec);
       W.exec = nullptr;
       cudaGraph_t graph = nullptr;
       e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-      for (int q = 0; q < kCheck && e == cudaSuccess; ++q) e = pcg_iteration<T>(P, a, launch, W, x, cs);
+      for (int q = 0; q < kCheck && e == cudaSuccess; ++q) e = iteration(q);
       const cudaError_t ec = cudaStreamEndCapture(cs, &graph);
       if (e == cudaSuccess) e = ec;
       if (e == cudaSuccess) e = cudaGraphInstantiate(&W.exec, graph, 0);
@@ -522,6 +699,7 @@ static cudaError_t pcg_core(const GsPlan &P, const AxArgs &base, cudaError_t (*l
         W.graph_x = x;
         W.graph_jac = W.jac;
         W.graph_op = base.geo;
+        W.graph_fused = fused;
       }
     }
     int issued = 0;
@@ -530,7 +708,7 @@ static cudaError_t pcg_core(const GsPlan &P, const AxArgs &base, cudaError_t (*l
       if (block == kCheck) {
         e = cudaGraphLaunch(W.exec, cs);
       } else {
-        for (int q = 0; q < block && e == cudaSuccess; ++q) e = pcg_iteration<T>(P, a, launch, W, x, cs);
+        for (int q = 0; q < block && e == cudaSuccess; ++q) e = iteration(q);  // after whole blocks: even
       }
       issued += block;
       if (e == cudaSuccess) e = cudaMemcpyAsync(hS, S, sizeof(double) * gs::kScalars, cudaMemcpyDeviceToHost, cs);
@@ -547,6 +725,10 @@ static cudaError_t pcg_core(const GsPlan &P, const AxArgs &base, cudaError_t (*l
         break;
       }
       it = issued;
+    }
+    if (e == cudaSuccess && fused && it > 0) {
+      gs::finish_x_kernel<T><<<gs::grid_for(n), 256, 0, cs>>>(n, S, (it & 1) ? W.w : W.p, x);
+      e = cudaGetLastError();
     }
     const cudaError_t e2 = cudaEventRecord(W.ev, cs);
     if (e2 == cudaSuccess) cudaStreamWaitEvent(s, W.ev, 0);
@@ -579,7 +761,7 @@ static cudaError_t cached_work(Ctx &ctx, int slot, PcgWork<T> **out) {
   if (!W) {
     W = new (std::nothrow) PcgWork<T>;
     if (!W) return cudaErrorMemoryAllocation;
-    cudaError_t e = W->alloc(ctx.gs.n_global, ctx.gs.n_local, true);
+    cudaError_t e = W->alloc(ctx.gs.n_global, ctx.gs.n_local, ctx.E);
     if (e != cudaSuccess) {
       delete_work<T>(W);
       return e;
@@ -683,8 +865,8 @@ struct MixedWork {
   PcgWork<float> W;
   double *r = nullptr, *w = nullptr, *Ul = nullptr, *Yl = nullptr, *S = nullptr, *part = nullptr, *hS = nullptr;
   float *r32 = nullptr, *d32 = nullptr;
-  cudaError_t alloc(int64_t n, int64_t nl) {
-    cudaError_t e = W.alloc(n, nl, true);
+  cudaError_t alloc(int64_t n, int64_t nl, int64_t E) {
+    cudaError_t e = W.alloc(n, nl, E);
     if (e == cudaSuccess) e = cudaMalloc(&r, sizeof(double) * n);
     if (e == cudaSuccess) e = cudaMalloc(&w, sizeof(double) * n);
     if (e == cudaSuccess) e = cudaMalloc(&Ul, sizeof(double) * nl);
@@ -729,7 +911,7 @@ cudaError_t pcg_mixed_run(Ctx &ctx, const AxArgs &hi, cudaError_t (*launch_hi)(c
   if (!MW) {
     MW = new (std::nothrow) MixedWork;
     if (!MW) return cudaErrorMemoryAllocation;
-    e = MW->alloc(n, nl);
+    e = MW->alloc(n, nl, ctx.E);
     if (e != cudaSuccess) {
       delete_mixed(MW);
       return e;

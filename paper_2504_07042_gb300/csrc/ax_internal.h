@@ -34,6 +34,12 @@ struct GsPlan {
   gidx *off = nullptr;  // [n_global + 1]
   gidx *idx = nullptr;  // [n_local], local indices grouped by global node, increasing within a group
   gidx *gid = nullptr;  // [n_local], global id of every local node
+  bool complete = false;  // every global node has a local copy
+  // The fused CG iteration's view of the same map (gs_fused_view, built by the
+  // first solve that runs it): own[m] = gid[m], sign bit set where m is the
+  // first local copy of its node; rank[idx[q]] = q, the place of a local copy
+  // among those of all nodes.
+  mutable gidx *own = nullptr, *rank = nullptr;
   uint8_t *mask = nullptr; // [n_global] Dirichlet mask or nullptr
 };
 
@@ -74,6 +80,20 @@ struct Ctx {
   std::string err;
 };
 
+// Operands of an AxLocal that is one half of a CG iteration (ax_gs.cu): X is
+// the new search direction, formed while it is loaded, and the kernel leaves
+// alpha.  Vectors in the context's value type, all of the assembled system; Y
+// goes to its nodes' places, Y[rank[m]], so that a node's copies lie together.
+struct CgArgs {
+  const gidx *own = nullptr, *rank = nullptr;  // [n_local] (GsPlan)
+  const void *z = nullptr;                  // preconditioned residual
+  const void *p = nullptr;                  // direction of the last iteration
+  void *pn = nullptr, *x = nullptr;         // direction of this one; solution
+  void *U = nullptr;                        // [n_local] the direction's local copies (float64 IO only)
+  double *S = nullptr, *part = nullptr;     // scalars; one partial sum per CTA
+  unsigned *cnt = nullptr;
+};
+
 // Argument bundle handed to every AxLocal launcher.
 struct AxArgs {
   int64_t E = 0;
@@ -86,6 +106,7 @@ struct AxArgs {
   cudaStream_t stream = nullptr;
   int tile = 0;      // tile variant (elements per CTA: 0 = base, 1 = twice; FP32 only)
   int64_t grid = 0;  // CTAs to launch (0 = one per block of elements; fewer = persistent loop)
+  const CgArgs *cg = nullptr;  // FP32 and double-word launchers: the CG form (E = 0 only prepares the kernel)
   // kernels with bounded waits (tensor-core AxLocal): error word, nonzero
   // once a wait ran out (read by the context's synchronising calls)
   int *err = nullptr;
@@ -133,6 +154,9 @@ cudaError_t setup_diag(const Ctx &c, const double *vertices, void *diag, bool f6
 // Gather-scatter and CG (ax_gs.cu).
 cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int64_t n_global, const uint8_t *mask_dev,
                      cudaStream_t s, int64_t *bad_ids);
+// Whether the fused CG iteration can run on the plan, building own and rank
+// on stream s if they are not there yet (false too when there is no room).
+bool gs_fused_view(const GsPlan &plan, cudaStream_t s);
 void gs_free(GsPlan &plan);
 cudaError_t gs_assemble_run(const GsPlan &p, bool f64, void *Y, cudaStream_t s);
 cudaError_t gs_gather_run(const GsPlan &p, bool f64, const void *Y, void *y, cudaStream_t s);

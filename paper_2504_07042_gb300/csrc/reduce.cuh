@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace ax {
 namespace red {
 
@@ -26,33 +28,81 @@ __device__ __forceinline__ void block_reduce_store(double v, double *out) {
 }
 
 // Fixed-order block reduction of two values at once, out_a[blockIdx.x] and
-// out_b[blockIdx.x]: the warp-level tree in the values' own type T (float
-// sums stay on the FP32 pipe; GB300's FP64 rate is 1/64 of it), the eight
-// warp results in double.  One CTA barrier.
+// out_b[blockIdx.x], one CTA barrier.  Float: the warp-level tree stays on the
+// FP32 pipe, the eight warp results are added in double.  Double: an addition
+// costs a warp 64 cycles of its SM quarter's FP64 pipe whatever its lanes do,
+// and a tree in every warp is 10 of them; through shared memory one warp adds
+// up all of a's threads and another all of b's, 13 each for the whole block.
 template <typename T>
 __device__ __forceinline__ void block_reduce2_store(T a, T b, double *out_a, double *out_b) {
-  __shared__ double sh[2][kThreads / 32];
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    sh[0][wid] = (double)a;
-    sh[1][wid] = (double)b;
-  }
-  __syncthreads();
-  if (wid == 0) {
-    double va = lane < kThreads / 32 ? sh[0][lane] : 0.0, vb = lane < kThreads / 32 ? sh[1][lane] : 0.0;
-    for (int o = kThreads / 64; o > 0; o >>= 1) {
-      va += __shfl_down_sync(0xffffffffu, va, o);
-      vb += __shfl_down_sync(0xffffffffu, vb, o);
+  if constexpr (sizeof(T) == 8) {
+    __shared__ double sh[2][kThreads];
+    sh[0][threadIdx.x] = a;
+    sh[1][threadIdx.x] = b;
+    __syncthreads();
+    if (wid == 0 || (wid == 1 && out_b)) {
+      double v = sh[wid][lane];
+      for (int q = lane + 32; q < kThreads; q += 32) v += sh[wid][q];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if (lane == 0) *(wid == 0 ? out_a : out_b) = v;
+    }
+  } else {
+    __shared__ double sh[2][kThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, o);
+      b += __shfl_down_sync(0xffffffffu, b, o);
     }
     if (lane == 0) {
-      *out_a = va;
-      if (out_b) *out_b = vb;
+      sh[0][wid] = (double)a;
+      sh[1][wid] = (double)b;
+    }
+    __syncthreads();
+    if (wid == 0) {
+      double va = lane < kThreads / 32 ? sh[0][lane] : 0.0, vb = lane < kThreads / 32 ? sh[1][lane] : 0.0;
+      for (int o = kThreads / 64; o > 0; o >>= 1) {
+        va += __shfl_down_sync(0xffffffffu, va, o);
+        vb += __shfl_down_sync(0xffffffffu, vb, o);
+      }
+      if (lane == 0) {
+        *out_a = va;
+        if (out_b) *out_b = vb;
+      }
     }
   }
+}
+
+// s[u] = the sum of node u's local copies, which lie together: c[u] of them at
+// Y[b[u]] on (c = 0: nothing, s = 0), in order.  The copies of all U nodes are
+// loaded together, one, one more (the copy across a face), then two at a time
+// (edges, corners); an addition is issued only where some lane of the warp
+// needs it: in float64 one that no lane needs would cost as much of GB300's
+// FP64 pipe (2 per clock and SM) as one that all need.
+template <typename T, int U, typename I>
+__device__ __forceinline__ void gather_copies(const T *Y, const I b[U], const I c[U], T s[U]) {
+  int top[U], most = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) s[u] = c[u] > 0 ? __ldcg(Y + b[u]) : T(0);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    top[u] = __reduce_max_sync(0xffffffffu, (int)c[u]);
+    most = max(most, top[u]);
+  }
+  auto step = [&](int q0, auto cnt) {
+    constexpr int n = decltype(cnt)::value;
+    T v[U][n];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < n; ++q) v[u][q] = q0 + q < c[u] ? __ldcg(Y + b[u] + q0 + q) : T(0);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int q = 0; q < n; ++q)
+        if (q0 + q < top[u]) s[u] += v[u][q];
+  };
+  if (most > 1) step(1, std::integral_constant<int, 1>{});
+  for (int q0 = 2; q0 < most; q0 += 2) step(q0, std::integral_constant<int, 2>{});
 }
 
 // Returns true in the block that arrives last at *cnt (after every block has
