@@ -278,9 +278,10 @@ ax_status ax_batch_set_wait(ax_batch *b, int64_t budget_ns, int stuck_mesh);
  *   batch is captured once as a CUDA graph and launched once per iteration
  *   (per-mesh scalars, segmented reductions, converged meshes idle).  In
  *   the persistent mode the graph holds ONE kernel: a queue of AxLocal
- *   tiles (the scatter fused into their loads), gather + dot, update and
- *   direction chunks, each waiting (bounded) for its mesh's previous phase;
- *   a wait past its budget stops the solve with AX_ETIMEOUT.
+ *   tiles (direction and update of x fused into their loads) and gather +
+ *   update chunks, each waiting (bounded) for its mesh's previous phase;
+ *   a wait past its budget stops the solve with AX_ETIMEOUT.  (A batch with a
+ *   node that no element has runs one launch per order group and phase.)
  *   graph = 0: reference path, each mesh solved in turn with its own
  *   launches (pcg_solve on its per-mesh context).
  *   iters, relres: host arrays [B].  AX_ENOTCONV if a mesh hit maxit.

@@ -171,6 +171,19 @@ __global__ void __launch_bounds__(kThreads)
   block_sum((double)bb, pbb + blockIdx.x);
 }
 
+// x += alpha p after a mesh's last iteration: the update that the fused
+// iteration still owes (p: the direction of odd or even iterations)
+__global__ void __launch_bounds__(kThreads)
+    seg_finish_x(Seg sg, const double *__restrict__ S, const float *__restrict__ p_even,
+                 const float *__restrict__ p_odd, float *__restrict__ x) {
+  const int m = sg.bmesh[blockIdx.x];
+  const int it = (int)S[m * kS + 9];
+  if (it == 0) return;
+  const float alpha = (float)S[m * kS + 10];
+  const float *p = (it & 1) ? p_odd : p_even;
+  for (int64_t g = sg.blo[blockIdx.x] + threadIdx.x; g < sg.bhi[blockIdx.x]; g += kThreads) x[g] += alpha * p[g];
+}
+
 // per mesh after the init reductions: tol^2, done when already converged
 __global__ void seg_start(int B, double *S, double rtol) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -743,41 +756,51 @@ ax_status batch_pcg(ax_batch *b, const T *bvec, T *x, double rtol, int maxit, in
     seg_start<<<(B + 127) / 128, 128, 0, s>>>(B, W.S, rtol);
     e = cudaGetLastError();
   }
-  // capture one iteration: one persistent launch (float32, N <= 9) or the
-  // per-phase launches
-  const bool one_launch = sizeof(T) == 4 && b->use_persist;
-  persist::Vecs pv;
+  // capture one iteration: one persistent launch (float32, N <= 9, every node
+  // with a local copy), once for each order of the two direction vectors, or
+  // the per-phase launches
+  const bool one_launch = sizeof(T) == 4 && b->use_persist && e == cudaSuccess && gs_fused_view(P, s);
+  double *part_ax = nullptr;
+  persist::Vecs pv[2];
   if (one_launch) {
-    pv.p = (float *)W.p;
-    pv.z = (float *)W.z;
-    pv.r = (float *)W.r;
-    pv.x = (float *)x;
-    pv.w = (float *)W.w;
-    pv.Yl = (float *)W.Yl;
-    pv.inv = (const float *)W.inv;
-    pv.gid = P.gid;
-    pv.off = P.off;
-    pv.idx = P.idx;
-    pv.mask = P.mask;
-    pv.S = W.S;
-    pv.part = W.part;
+    if (e == cudaSuccess) e = cudaMalloc(&part_ax, sizeof(double) * std::max(1, b->ps->sc.n_ax));
+    for (int q = 0; q < 2; ++q) {
+      persist::Vecs &v = pv[q];
+      v.p = (float *)(q ? W.w : W.p);
+      v.pn = (float *)(q ? W.p : W.w);
+      v.r = (float *)W.r;
+      v.z = (float *)W.z;
+      v.x = (float *)x;
+      v.Yl = (float *)W.Yl;
+      v.inv = (const float *)W.inv;
+      v.own = P.own;
+      v.rank = P.rank;
+      v.off = P.off;
+      v.mask = P.mask;
+      v.S = W.S;
+      v.part = W.part;
+      v.part_ax = part_ax;
+    }
     if (e == cudaSuccess) e = persist::plan_reset(*b->ps, s);
   }
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t gexec = nullptr;
-  if (e == cudaSuccess) e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    cudaError_t e2 = one_launch ? persist::launch_iteration(*b->ps, pv, s) : batch_iteration<T>(b, W, x, s);
-    e = cudaStreamEndCapture(s, &graph);
-    if (e == cudaSuccess) e = e2;
+  cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+  for (int q = 0; q < (one_launch ? 2 : 1) && e == cudaSuccess; ++q) {
+    cudaGraph_t graph = nullptr;
+    e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+      const cudaError_t e2 = one_launch ? persist::launch_iteration(*b->ps, pv[q], s) : batch_iteration<T>(b, W, x, s);
+      e = cudaStreamEndCapture(s, &graph);
+      if (e == cudaSuccess) e = e2;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&gexec[q], graph, 0);
+    if (graph) cudaGraphDestroy(graph);
   }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&gexec, graph, 0);
   int issued = 0;
   bool all_done = false;
   int pstatus = 0;  // persistent kernel: status word (AX_ETIMEOUT after a wait ran out)
   while (e == cudaSuccess && issued < maxit && !all_done && pstatus == 0) {
     const int block = std::min(16, maxit - issued);
-    for (int q = 0; q < block && e == cudaSuccess; ++q) e = cudaGraphLaunch(gexec, s);
+    for (int q = 0; q < block && e == cudaSuccess; ++q) e = cudaGraphLaunch(gexec[one_launch ? (issued + q) & 1 : 0], s);
     issued += block;
     if (e == cudaSuccess) e = cudaMemcpyAsync(W.hS, W.S, sizeof(double) * kS * B, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && one_launch)
@@ -788,6 +811,7 @@ ax_status batch_pcg(ax_batch *b, const T *bvec, T *x, double rtol, int maxit, in
       if (W.hS[m * kS + 6] == 0.0) all_done = false;
   }
   if (e == cudaSuccess) {
+    if (one_launch) seg_finish_x<<<RB, kThreads, 0, s>>>(sg, W.S, (const float *)W.p, (const float *)W.w, (float *)x);
     e = cudaMemcpyAsync(W.hS, W.S, sizeof(double) * kS * B, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
@@ -804,13 +828,13 @@ ax_status batch_pcg(ax_batch *b, const T *bvec, T *x, double rtol, int maxit, in
     e = persist::plan_reset(*b->ps, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  if (gexec) cudaGraphExecDestroy(gexec);
-  if (graph) cudaGraphDestroy(graph);
+  for (cudaGraphExec_t g : gexec)
+    if (g) cudaGraphExecDestroy(g);
   if (e == cudaSuccess) e = cudaEventRecord(ev, s);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(user, ev, 0);
   if (ev) cudaEventDestroy(ev);
   cudaFree(W.r); cudaFree(W.z); cudaFree(W.p); cudaFree(W.w); cudaFree(W.inv); cudaFree(W.Ul); cudaFree(W.Yl);
-  cudaFree(W.dl); cudaFree(W.S); cudaFree(W.part); cudaFreeHost(W.hS);
+  cudaFree(W.dl); cudaFree(W.S); cudaFree(W.part); cudaFree(part_ax); cudaFreeHost(W.hS);
   if (e != cudaSuccess) return bcuda(b, e, "ax_batch_pcg");
   if (pstatus != 0)
     return bfail(b, AX_ETIMEOUT,

@@ -742,15 +742,6 @@ struct XDirect {
   const IO *__restrict__ p;
   __device__ __forceinline__ IO operator[](int64_t m) const { return p[m]; }
 };
-// The local copies of a global vector, X[m] = u[gid[m]].
-template <typename IO>
-struct XGather {
-  static constexpr bool kCg = false;
-  const IO *__restrict__ u;
-  const gidx *__restrict__ gid;
-  __device__ __forceinline__ IO operator[](int64_t m) const { return u[gid[m]]; }
-};
-
 // The search direction of a CG iteration, formed at each local copy while it
 // is loaded: p_new[g] = z[g] + beta p[g].  The thread that loads a node's
 // first copy also stores p_new and brings x up to date, x += alpha p, with

@@ -9,15 +9,17 @@
 // part in the barriers only).
 //
 // One CG iteration of every mesh of the batch (Eq. 1: A = Q^T blkdiag(A^e) Q,
-// Jacobi-preconditioned) is the same kernel with four kinds of items, queued
-// phase after phase:
-//   AX  AxLocal tiles, X read as the local copies of the search direction
-//       (X[m] = p[gid[m]]: the scatter Q p fused into the load)
-//   GD  chunks of global nodes: w = mask(Q^T Y), partial p.w; the last chunk
-//       of a mesh to finish sums the partials in a fixed order and sets alpha
-//   UP  chunks: x += alpha p, r -= alpha w, z = D^-1 r, partial r.z, r.r; the
-//       last one sets beta, counts the iteration and tests convergence
-//   DI  chunks: p = z + beta p
+// Jacobi-preconditioned) is the same kernel with two kinds of items, queued
+// one after the other (the fused iteration of ax_gs.cu, per mesh):
+//   AX  AxLocal tiles, X formed while it is loaded: p_new = z + beta p at the
+//       local copies, x += alpha p where a node's first copy lies; partial
+//       p . A p over the local copies; the last tile of a mesh to finish sums
+//       the partials in a fixed order and sets alpha
+//   GU  chunks of global nodes: r -= alpha Q^T Y, z = D^-1 r, partial r.z and
+//       r.r; the last one sets beta, counts the iteration and tests convergence
+// (With four kinds of items, gather and dot, update, and direction apart from
+// each other, and w and the scatter of p through memory between them, 16 meshes
+// (7.7e6 local nodes) took 250 us per iteration on GB300 instead of 182.)
 // An item waits (thread 0, bounded spin on a per-mesh arrival counter) until
 // the items of the previous phase of its mesh have arrived.  Items are
 // dequeued in queue order and an item only waits on items queued before it,
@@ -34,6 +36,7 @@
 
 #include "ax_internal.h"
 #include "ax_persist.h"
+#include "reduce.cuh"
 
 // float32 tables of this translation unit (no per-order launcher)
 #define AX_POLICY fiber::Native<float>
@@ -47,7 +50,7 @@ namespace persist {
 
 using P = fiber::Native<float>;
 constexpr int kS = 16;  // per-mesh scalars, same slots as the batched CG of ax_batch.cu
-constexpr int kU = 4;   // gather-dot: nodes per thread whose gathers are in flight together
+constexpr int kU = 4;   // gather-update: nodes per thread whose gathers are in flight together
 
 __device__ __forceinline__ unsigned long long now_ns() {
   unsigned long long t;
@@ -125,167 +128,148 @@ __device__ double cta_sum(double v) {
 }
 
 // One AxLocal tile: elements [e0, e0 + cnt) of group g, in blocks of EPB.
+// Returns this thread's share of X . Y in the CG form (x: see XCg), else 0.
 // Not inlined: each order keeps its own register allocation (inlined into
 // one body, the nine orders' code took every register there is).
 template <int N1, int KIND, bool PCG>
-__device__ __noinline__ void ax_tile(unsigned char *smem, const Group &g, int64_t e0, int cnt, const float *X, const float *p,
-                        const gidx *gid, float *Y) {
+__device__ __noinline__ float ax_tile(unsigned char *smem, const Group &g, int64_t e0, int cnt, const float *X,
+                                      const fiber::XCg<float> *x, float *Y) {
   using Sh = fiber::Shape<N1, 1, 0>;
   using Buf = fiber::FiberSmem<P, N1, KIND, 1, 0>;
   static_assert(Sh::threads <= kThreads, "order shape wider than the persistent CTA");
   const Buf sm = Buf::carve(smem);
   const int tid = threadIdx.x;
-  float *Yg = Y + g.loc;
+  float *Yg = PCG ? Y : Y + g.loc;  // the CG form stores Y by rank over the whole batch
+  float xy = 0.0f;
   for (int64_t b = e0; b < e0 + cnt; b += Sh::EPB) {
     const int nel = (int)((e0 + cnt - b) < Sh::EPB ? (e0 + cnt - b) : Sh::EPB);
     if constexpr (PCG) {
-      fiber::fiber_block<P, N1, KIND, 1, true, fiber::XGather<float>, 0>(
-          sm, tid, b, nel, (const float *)g.geo, (const float *)g.lam, fiber::XGather<float>{p, gid + g.loc}, Yg);
+      fiber::XCg<float> xg = *x;
+      xg.own += g.loc;
+      xg.rank += g.loc;
+      xy += fiber::fiber_block<P, N1, KIND, 1, true, fiber::XCg<float>, 0>(sm, tid, b, nel, (const float *)g.geo,
+                                                                           (const float *)g.lam, xg, Yg);
     } else {
       fiber::fiber_block<P, N1, KIND, 1, true, fiber::XDirect<float>, 0>(
           sm, tid, b, nel, (const float *)g.geo, (const float *)g.lam, fiber::XDirect<float>{X + g.loc}, Yg);
     }
   }
+  return xy;
 }
 
 template <int KIND, bool PCG>
 __device__ void run_ax(unsigned char *smem, const Sched &sc, const Vecs &v, int item, const float *X, float *Y) {
   const AxItem t = sc.ax[item];
   const Group g = sc.groups[t.group];
-  const bool skip = PCG && __ldcg(&v.S[t.mesh * kS + 6]) != 0.0;  // mesh converged in an earlier launch
+  double *S = PCG ? v.S + t.mesh * kS : nullptr;
+  const bool skip = PCG && __ldcg(S + 6) != 0.0;  // mesh converged in an earlier launch
+  float xy = 0.0f;
   if (!skip) {
+    fiber::XCg<float> x{};
+    if constexpr (PCG)
+      x = fiber::XCg<float>{v.own, v.rank, v.z, v.p, v.pn, v.x, nullptr, (float)__ldcg(S + 10), (float)__ldcg(S + 11)};
     switch (g.N1) {
 #define PX_CASE(n1) \
-  case n1: ax_tile<n1, KIND, PCG>(smem, g, t.e0, t.cnt, X, v.p, v.gid, Y); break;
+  case n1: xy = ax_tile<n1, KIND, PCG>(smem, g, t.e0, t.cnt, X, &x, Y); break;
       PX_CASE(2) PX_CASE(3) PX_CASE(4) PX_CASE(5) PX_CASE(6) PX_CASE(7) PX_CASE(8) PX_CASE(9) PX_CASE(10)
 #undef PX_CASE
       default: break;
     }
   }
-  if (PCG) cta_arrive(&sc.cnt[t.mesh], 1 << 30);
+  if constexpr (PCG) {
+    const double s = cta_sum((double)xy);
+    if (threadIdx.x == 0) v.part_ax[item] = s;
+    const int need = sc.ax_need[t.mesh];
+    if (cta_arrive(&sc.cnt[t.mesh], need)) {
+      double a = 0.0;
+      const int lo = sc.ax_beg[t.mesh];
+      for (int q = lo + threadIdx.x; q < lo + need; q += kThreads) a += __ldcg(&v.part_ax[q]);
+      a = cta_sum(a);
+      if (threadIdx.x == 0 && !skip) {
+        S[1] = a;
+        S[10] = a != 0.0 ? __ldcg(S) / a : 0.0;
+      }
+      cta_arrive(&sc.cnt[t.mesh], 1 << 30);  // need + 1: alpha is set
+    }
+  }
 }
 
-// GD: w = mask(Q^T Y) on the chunk, partial p.w; the mesh's last chunk sets
-// S[1] = p.w and alpha = S[0] / p.w (slot 10).
-__device__ void run_gd(const Sched &sc, const Vecs &v, int c) {
+// GU: r -= alpha Q^T Y on the chunk, partial r.z and r.r; the mesh's last
+// chunk sets r.z (slot 4), r.r (slot 2), beta (slot 11), counts the iteration
+// and tests convergence (the batched CG's seg_check).
+__device__ void run_gu(const Sched &sc, const Vecs &v, int c) {
   const int m = sc.cmesh[c];
   const int stuck = m == sc.stuck_mesh ? 1 : 0;  // test hook: a dependency nothing completes
-  if (!cta_wait(&sc.cnt[m], sc.ax_need[m] + stuck, sc)) return;
-  const bool done = __ldcg(&v.S[m * kS + 6]) != 0.0;
-  float d = 0.0f;
+  if (!cta_wait(&sc.cnt[m], sc.ax_need[m] + 1 + stuck, sc)) return;
+  double *S = v.S + m * kS;
+  const bool done = __ldcg(S + 6) != 0.0;
+  float rz = 0.0f, rr = 0.0f;
   if (!done) {
-    // kU nodes per thread at a time, their gathers issued together (a hexahedral
-    // node has at most 8 local copies; more are summed by the tail loop)
+    const float alpha = (float)__ldcg(S + 10);
+    // kU nodes per thread at a time, their loads issued together
     const int64_t hi = sc.chi[c];
-    for (int64_t g0 = sc.clo[c] + threadIdx.x; g0 < hi; g0 += kU * kThreads) {
+    for (int64_t base = sc.clo[c]; base < hi; base += kU * kThreads) {
+      const int64_t g0 = base + threadIdx.x;
       gidx b[kU], n[kU];
-      float s[kU];
+      float s[kU], rv[kU], iv[kU];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         const int64_t g = g0 + u * kThreads;
-        b[u] = g < hi ? v.off[g] : 0;
-        n[u] = g < hi ? v.off[g + 1] - b[u] : 0;
-        s[u] = 0.0f;
+        const bool on = g < hi;
+        b[u] = on ? v.off[g] : 0;
+        n[u] = on ? v.off[g + 1] - b[u] : 0;
+        rv[u] = on ? v.r[g] : 0.0f;
+        iv[u] = on ? v.inv[g] : 0.0f;
       }
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-          if (q < n[u]) s[u] += __ldcg(&v.Yl[v.idx[b[u] + q]]);
+      red::gather_copies<float, kU>(v.Yl, b, n, s);
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         const int64_t g = g0 + u * kThreads;
         if (g >= hi) break;
-        for (int q = 8; q < n[u]; ++q) s[u] += __ldcg(&v.Yl[v.idx[b[u] + q]]);
-        if (v.mask && v.mask[g]) s[u] = 0.0f;
-        v.w[g] = s[u];
-        d += v.p[g] * s[u];
+        const bool mk = v.mask && v.mask[g];
+        if (mk) s[u] = 0.0f;
+        const float rg = rv[u] - alpha * s[u];
+        const float zg = mk ? 0.0f : rg * iv[u];
+        v.r[g] = rg;
+        v.z[g] = zg;
+        rz += rg * zg;
+        rr += rg * rg;
       }
-    }
-  }
-  const double ds = cta_sum((double)d);
-  if (threadIdx.x == 0) v.part[c] = ds;
-  const int need = sc.pbeg[m + 1] - sc.pbeg[m];
-  if (cta_arrive(&sc.cnt[sc.B + m], need)) {
-    double s = 0.0;
-    for (int q = sc.pbeg[m] + threadIdx.x; q < sc.pbeg[m + 1]; q += kThreads) s += __ldcg(&v.part[q]);
-    s = cta_sum(s);
-    if (threadIdx.x == 0 && !done) {
-      v.S[m * kS + 1] = s;
-      v.S[m * kS + 10] = s != 0.0 ? __ldcg(&v.S[m * kS + 0]) / s : 0.0;
-    }
-    cta_arrive(&sc.cnt[sc.B + m], 1 << 30);  // need + 1: alpha is set
-  }
-}
-
-// UP: x, r, z on the chunk, partial r.z and r.r; the mesh's last chunk sets
-// r.z (slot 4), r.r (slot 2), beta (slot 11), counts the iteration and tests
-// convergence (the batched CG's seg_check).
-__device__ void run_up(const Sched &sc, const Vecs &v, int c) {
-  const int m = sc.cmesh[c];
-  const int need = sc.pbeg[m + 1] - sc.pbeg[m];
-  if (!cta_wait(&sc.cnt[sc.B + m], need + 1, sc)) return;
-  const bool done = __ldcg(&v.S[m * kS + 6]) != 0.0;
-  float rz = 0.0f, rr = 0.0f;
-  if (!done) {
-    const float alpha = (float)__ldcg(&v.S[m * kS + 10]);
-#pragma unroll 4
-    for (int64_t g = sc.clo[c] + threadIdx.x; g < sc.chi[c]; g += kThreads) {
-      const float rg = v.r[g] - alpha * __ldcg(&v.w[g]);
-      float zg = v.inv ? rg * v.inv[g] : rg;
-      if (v.mask && v.mask[g]) zg = 0.0f;
-      v.x[g] += alpha * v.p[g];
-      v.r[g] = rg;
-      v.z[g] = zg;
-      rz += rg * zg;
-      rr += rg * rg;
     }
   }
   const double rzs = cta_sum((double)rz);
   const double rrs = cta_sum((double)rr);
   if (threadIdx.x == 0) {
-    v.part[sc.n_chunks + c] = rzs;
-    v.part[2 * sc.n_chunks + c] = rrs;
+    v.part[c] = rzs;
+    v.part[sc.n_chunks + c] = rrs;
   }
-  if (cta_arrive(&sc.cnt[2 * sc.B + m], need)) {
+  const int need = sc.pbeg[m + 1] - sc.pbeg[m];
+  if (cta_arrive(&sc.cnt[sc.B + m], need)) {
     double a = 0.0, b = 0.0;
     for (int q = sc.pbeg[m] + threadIdx.x; q < sc.pbeg[m + 1]; q += kThreads) {
-      a += __ldcg(&v.part[sc.n_chunks + q]);
-      b += __ldcg(&v.part[2 * sc.n_chunks + q]);
+      a += __ldcg(&v.part[q]);
+      b += __ldcg(&v.part[sc.n_chunks + q]);
     }
     a = cta_sum(a);
     b = cta_sum(b);
     if (threadIdx.x == 0 && !done) {
-      double *s = v.S + m * kS;
-      s[4] = a;
-      s[2] = b;
-      const double s0 = __ldcg(&s[0]);
-      s[11] = s0 != 0.0 ? a / s0 : 0.0;
-      const double it = __ldcg(&s[9]) + 1.0;
-      s[9] = it;
-      if (b <= __ldcg(&s[8])) {
-        s[6] = 1.0;
-        s[7] = it;
+      S[4] = a;
+      S[2] = b;
+      const double s0 = __ldcg(S);
+      S[11] = s0 != 0.0 ? a / s0 : 0.0;
+      const double it = __ldcg(S + 9) + 1.0;
+      S[9] = it;
+      if (b <= __ldcg(S + 8)) {
+        S[6] = 1.0;
+        S[7] = it;
       } else if (!(b == b)) {
-        s[6] = 1.0;
-        s[7] = -it;
+        S[6] = 1.0;
+        S[7] = -it;
       } else {
-        s[0] = a;
+        S[0] = a;
       }
     }
-    cta_arrive(&sc.cnt[2 * sc.B + m], 1 << 30);  // need + 1: beta and the test are set
   }
-}
-
-// DI: p = z + beta p on the chunk (meshes that converged keep p)
-__device__ void run_di(const Sched &sc, const Vecs &v, int c) {
-  const int m = sc.cmesh[c];
-  const int need = sc.pbeg[m + 1] - sc.pbeg[m];
-  if (!cta_wait(&sc.cnt[2 * sc.B + m], need + 1, sc)) return;
-  if (__ldcg(&v.S[m * kS + 6]) != 0.0) return;
-  const float beta = (float)__ldcg(&v.S[m * kS + 11]);
-#pragma unroll 4
-  for (int64_t g = sc.clo[c] + threadIdx.x; g < sc.chi[c]; g += kThreads) v.p[g] = __ldcg(&v.z[g]) + beta * v.p[g];
 }
 
 // Resident CTAs the register budget is sized for (64 registers a thread, as
@@ -293,13 +277,13 @@ __device__ void run_di(const Sched &sc, const Vecs &v, int c) {
 constexpr int kMinCtasPersist = 8;
 
 // The persistent kernel.  PCG false: AX items only, X and Y given.  PCG
-// true: one CG iteration of every mesh (AX, GD, UP, DI items).
+// true: one CG iteration of every mesh (AX and GU items).
 template <int KIND, bool PCG>
 __global__ void __launch_bounds__(kThreads, kMinCtasPersist) persist_kernel(Sched sc, Vecs v, const float *__restrict__ X,
                                                            float *__restrict__ Y) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
-  const int total = sc.n_ax + (PCG ? 3 * sc.n_chunks : 0);
+  const int total = sc.n_ax + (PCG ? sc.n_chunks : 0);
   for (;;) {
     if (threadIdx.x == 0) s_item = *(volatile int *)sc.abortf ? total : atomicAdd(sc.ticket, 1);
     __syncthreads();
@@ -309,13 +293,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPersist) persist_kernel(Sche
     if (it < sc.n_ax) {
       run_ax<KIND, PCG>(smem, sc, v, it, X, PCG ? v.Yl : Y);
     } else if (PCG) {
-      const int k = it - sc.n_ax, ph = k / sc.n_chunks, c = k - ph * sc.n_chunks;
-      if (ph == 0)
-        run_gd(sc, v, c);
-      else if (ph == 1)
-        run_up(sc, v, c);
-      else
-        run_di(sc, v, c);
+      run_gu(sc, v, it - sc.n_ax);
     }
   }
   // the last CTA out resets the queue for the next launch
@@ -323,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, kMinCtasPersist) persist_kernel(Sche
     __threadfence();
     if (atomicAdd(sc.exitc, 1) == (int)gridDim.x - 1) {
       *sc.ticket = 0;
-      for (int q = 0; q < 3 * sc.B; ++q) sc.cnt[q] = 0;
+      for (int q = 0; q < 2 * sc.B; ++q) sc.cnt[q] = 0;
       __threadfence();
       *sc.exitc = 0;
     }
@@ -429,7 +407,7 @@ cudaError_t plan_build(Plan &pl, cudaStream_t s) {
   // items: per mesh, tiles of tile_blocks x EPB elements; larger orders first
   // (longer items), meshes in batch order within an order
   std::vector<AxItem> items;
-  std::vector<int> need(pl.B, 0);
+  std::vector<int> need(pl.B, 0), beg(pl.B, 0);  // a mesh's items follow one another
   std::vector<int> gorder(pl.groups.size());
   for (size_t g = 0; g < gorder.size(); ++g) gorder[g] = (int)g;
   std::stable_sort(gorder.begin(), gorder.end(), [&](int a, int b) { return pl.groups[a].N1 > pl.groups[b].N1; });
@@ -437,6 +415,7 @@ cudaError_t plan_build(Plan &pl, cudaStream_t s) {
     const int64_t tile = (int64_t)pl.tile_blocks[g] * epb_of(pl.groups[g].N1);
     for (int m = 0; m < pl.B; ++m) {
       if (pl.mesh_group[m] != g) continue;
+      beg[m] = (int)items.size();
       for (int64_t a = 0; a < pl.mesh_E[m]; a += tile) {
         AxItem it;
         it.group = g;
@@ -473,14 +452,16 @@ cudaError_t plan_build(Plan &pl, cudaStream_t s) {
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(pl.pbeg_d, pb.data(), sizeof(int) * pb.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMalloc(&pl.ax_d, sizeof(AxItem) * std::max<size_t>(1, items.size()));
-  if (e == cudaSuccess) e = cudaMalloc(&pl.ax_need_d, sizeof(int) * pl.B);
-  if (e == cudaSuccess) e = cudaMalloc(&pl.ctl_d, sizeof(int) * (4 + 3 * pl.B));
+  if (e == cudaSuccess) e = cudaMalloc(&pl.ax_need_d, sizeof(int) * 2 * pl.B);
+  if (e == cudaSuccess) e = cudaMalloc(&pl.ctl_d, sizeof(int) * (4 + 2 * pl.B));
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(pl.groups_d, pl.groups.data(), sizeof(Group) * pl.groups.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && !items.empty())
     e = cudaMemcpyAsync(pl.ax_d, items.data(), sizeof(AxItem) * items.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(pl.ax_need_d, need.data(), sizeof(int) * pl.B, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(pl.ctl_d, 0, sizeof(int) * (4 + 3 * pl.B), s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(pl.ax_need_d + pl.B, beg.data(), sizeof(int) * pl.B, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(pl.ctl_d, 0, sizeof(int) * (4 + 2 * pl.B), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host vectors go out of scope
   if (e != cudaSuccess) return e;
   pl.sc.B = pl.B;
@@ -493,6 +474,7 @@ cudaError_t plan_build(Plan &pl, cudaStream_t s) {
   pl.sc.ax = pl.ax_d;
   pl.sc.n_ax = (int)items.size();
   pl.sc.ax_need = pl.ax_need_d;
+  pl.sc.ax_beg = pl.ax_need_d + pl.B;
   pl.sc.ticket = pl.ctl_d;
   pl.sc.exitc = pl.ctl_d + 1;
   pl.sc.status = pl.ctl_d + 2;
@@ -519,7 +501,7 @@ cudaError_t launch_local(const Plan &pl, const float *X, float *Y, cudaStream_t 
 }
 
 cudaError_t launch_iteration(const Plan &pl, const Vecs &v, cudaStream_t s) {
-  const int total = pl.sc.n_ax + 3 * pl.sc.n_chunks;
+  const int total = pl.sc.n_ax + pl.sc.n_chunks;
   if (total == 0) return cudaSuccess;
   const int grid = std::min(plan_grid(pl), total);
   switch (pl.kind) {

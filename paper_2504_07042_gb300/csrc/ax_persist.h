@@ -42,25 +42,28 @@ struct Sched {
   const AxItem *ax = nullptr;
   int n_ax = 0;
   const int *ax_need = nullptr;  // [B] AxLocal items per mesh
+  const int *ax_beg = nullptr;   // [B] a mesh's first item (its items follow one another)
   // vector chunks (kChunk global nodes, never across meshes): chunk c covers
   // global nodes [clo[c], chi[c]) of mesh cmesh[c]; mesh m owns chunks [pbeg[m], pbeg[m+1])
   int n_chunks = 0;
   const int *cmesh = nullptr;
   const int64_t *clo = nullptr, *chi = nullptr;
   const int *pbeg = nullptr;
-  // control words (device, zero at rest): ticket, exit count, status, abort flag, then cnt[3][B]
+  // control words (device, zero at rest): ticket, exit count, status, abort flag, then cnt[2][B]
   int *ticket = nullptr, *exitc = nullptr, *status = nullptr, *abortf = nullptr, *cnt = nullptr;
   long long budget_ns = kDefaultBudgetNs;
   int stuck_mesh = -1;  // test hook: this mesh's chunks wait for one AxLocal item too many
 };
 
 // The CG state of the batch (float32 vectors; per-mesh scalars in S[m][16]).
+// p and pn (the last iteration's direction and this one's) change places from
+// launch to launch.
 struct Vecs {
-  float *p = nullptr, *z = nullptr, *r = nullptr, *x = nullptr, *w = nullptr, *Yl = nullptr;
+  float *p = nullptr, *pn = nullptr, *r = nullptr, *z = nullptr, *x = nullptr, *Yl = nullptr;
   const float *inv = nullptr;
-  const gidx *gid = nullptr, *off = nullptr, *idx = nullptr;
+  const gidx *own = nullptr, *rank = nullptr, *off = nullptr;
   const uint8_t *mask = nullptr;
-  double *S = nullptr, *part = nullptr;  // part: [3][n_chunks]
+  double *S = nullptr, *part = nullptr, *part_ax = nullptr;  // part: [2][n_chunks]; part_ax: [n_ax]
 };
 
 // Host-side plan of one batch.
