@@ -1225,7 +1225,7 @@ constexpr bool kHasCg = P::kRoll || sizeof(typename P::IO) == 4;
 // loads, x += alpha p, W = A_e p_new, and alpha = r.z / p.w by the CTA that
 // arrives last.  It takes the place of a direction-and-scatter kernel, the
 // plain AxLocal and a dot product; the vectors' loads overlap the arithmetic
-// that bounds the operator: order 7, 4096 elements, double-word 78 us (AxLocal
+// that bounds the operator: order 7, 4096 elements, double-word 75 us (AxLocal
 // alone 60), float32 20 (10); the kernels whose place it takes took 38 and 25.
 // (A resident CTA per slot that loops over the blocks keeps the CTAs' phases
 // in step: 86 us instead of 78.)
@@ -1376,7 +1376,10 @@ cudaError_t launch_ax_cg(const AxArgs &a) {
   using Sh = Shape<N1, 1, kEpb<P, N1, KIND>, kLayout<P, N1, KIND>>;
   static_assert(Sh::threads >= 32 && (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S) >= Sh::threads * sizeof(double),
                 "a whole warp and a double per thread for the sums");
-  static const size_t smem = launch_smem<P, N1, KIND, 1>((const void *)ax_fiber_cg_kernel<P, N1, KIND>);
+  // (no cap on the resident CTAs as in launch_smem: their registers keep them
+  // to five at N1 = 8, and what shared memory leaves of L1 serves the gathers:
+  // double-word iterations at order 7, 4096 elements 104 -> 100 us)
+  constexpr size_t smem = (size_t)3 * Sh::EPB * Sh::ES * sizeof(typename P::S);
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(ax_fiber_cg_kernel<P, N1, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
