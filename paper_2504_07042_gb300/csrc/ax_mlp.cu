@@ -72,6 +72,7 @@ struct GradSum {
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const __grid_constant__ GradSum a) {
   __shared__ float sh[8][32];
   const int tid = threadIdx.x;
+  tc::wait_previous();
   if ((int)blockIdx.x < a.nw) {
     int64_t i = ((int64_t)blockIdx.x * 256 + tid) * 4;  // over the three weight ranges, one after the other
     int p = 0;
@@ -672,8 +673,7 @@ cudaError_t forward_backward(ax_mlp *m, const __nv_bfloat16 *X, const float *T, 
   a.rows32 = (int)rows32;
   a.nsq = tc::gemm_tiles((int)M, kOut) * tc::kEpiWarps;
   a.nw = (int)((nw / 4 + 255) / 256);
-  grad_reduce_kernel<<<a.nw + 3 * (kHid / 32) + 1, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return tc::launch_after(grad_reduce_kernel, a.nw + 3 * (kHid / 32) + 1, 256, 0, s, a);
 }
 
 }  // namespace
