@@ -228,6 +228,14 @@ __device__ __forceinline__ void st_op(unsigned char *base, uint32_t off, float v
   st_code<OP>(base, off, code<OP>(v));
 }
 
+// The geometry at two nodes per instruction stream (fiber::Geometry2, the same
+// results): measured on GB300 at order 7 11 to 16% faster for the trilinear kind
+// (TF32 196 -> 217 GDOF/s), 21 to 29% for the partial, 2 to 11% for the
+// parallelepiped and 6 to 8% for the stored kind with 16-bit operands, but 3%
+// slower for the stored kind in TF32 (182 -> 176).
+template <int KIND, int OP>
+constexpr bool kPacked7 = !(KIND == AX_GEOM_STORED && OP == 0);
+
 template <int KIND, int OP>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm<KIND>)
     ax_umma_kernel(int64_t E, const float *__restrict__ geo, const float *__restrict__ lam,
@@ -370,29 +378,43 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm<KIND>)
     // 4. geometry along the t-fiber of (i, j) = (la, lb), element le
     uint32_t tt[8];  // the t values, coded in the operand format
     {
-      // two nodes per instruction stream (Geometry2); rows beyond the last
-      // element work on the tile's first one's geometry, their results are
-      // not stored
-      const int64_t e = le < nel ? e0 + le : e0;
+      // two nodes per instruction stream (Geometry2, kPacked7), where rows beyond
+      // the last element work on the tile's first one's geometry; their results
+      // are not stored
+      constexpr bool kPk = kPacked7<KIND, OP>;
+      const bool live = le < nel;
+      const int64_t e = !kPk || live ? e0 + le : e0;
       fiber::Geometry<P, kN1, KIND> gm;
       gm.template prologue<false>(sgeo + le * (GW > 0 ? GW : 1), cx, cw, la, lb,
-                                  KIND == AX_GEOM_STORED ? geo + e * 7 * kN3 : nullptr,
-                                  KIND == AX_GEOM_TRILINEAR_PARTIAL ? lam + e * kN3 : nullptr, nullptr);
-      const fiber::Geometry2<kN1, KIND> g2(gm);
+                                  (KIND == AX_GEOM_STORED && (kPk || live)) ? geo + e * 7 * kN3 : nullptr,
+                                  (KIND == AX_GEOM_TRILINEAR_PARTIAL && (kPk || live)) ? lam + e * kN3 : nullptr, nullptr);
+      // 5. r, s into their operand buffers at once (the forward MMAs are
+      // done and the exchange buffers are apart), t after the loop
+      auto put = [&](int k, float r, float s, float t) {
+        st_op<OP>(bufR, cm_off<ESZ>(lb + 8 * k + 64 * le, la, F::kLboR, F::kSboR), r);
+        st_op<OP>(bufS, cm_off<ESZ>(la + 8 * k + 64 * le, lb, F::kLboS, F::kSboS), s);
+        tt[k] = code<OP>(t);
+      };
+      if constexpr (kPk) {
+        const fiber::Geometry2<kN1, KIND> g2(gm);
 #pragma unroll
-      for (int k = 0; k < kN1 / 2; ++k) {
-        const int k2 = kN1 - 1 - k, o = xown + kXk * k, o2 = xown + kXk * k2, l = la + lb * kN1;
-        const float2 xv[3] = {make_float2(ex0[o], ex0[o2]), make_float2(ex1[o], ex1[o2]), make_float2(x2[k], x2[k2])};
-        float2 o3[3];
-        g2.apply(l + k * kN1 * kN1, l + k2 * kN1 * kN1, make_float2(cx[k], cx[k2]), cw[k], xv, o3);
-        // 5. r, s into their operand buffers at once (the forward MMAs are
-        // done and the exchange buffers are apart), t after the loop
-        st_op<OP>(bufR, cm_off<ESZ>(lb + 8 * k + 64 * le, la, F::kLboR, F::kSboR), o3[0].x);
-        st_op<OP>(bufR, cm_off<ESZ>(lb + 8 * k2 + 64 * le, la, F::kLboR, F::kSboR), o3[0].y);
-        st_op<OP>(bufS, cm_off<ESZ>(la + 8 * k + 64 * le, lb, F::kLboS, F::kSboS), o3[1].x);
-        st_op<OP>(bufS, cm_off<ESZ>(la + 8 * k2 + 64 * le, lb, F::kLboS, F::kSboS), o3[1].y);
-        tt[k] = code<OP>(o3[2].x);
-        tt[k2] = code<OP>(o3[2].y);
+        for (int k = 0; k < kN1 / 2; ++k) {
+          const int k2 = kN1 - 1 - k, o = xown + kXk * k, o2 = xown + kXk * k2, l = la + lb * kN1;
+          const float2 xv[3] = {make_float2(ex0[o], ex0[o2]), make_float2(ex1[o], ex1[o2]), make_float2(x2[k], x2[k2])};
+          float2 o3[3];
+          g2.apply(l + k * kN1 * kN1, l + k2 * kN1 * kN1, make_float2(cx[k], cx[k2]), cw[k], xv, o3);
+          put(k, o3[0].x, o3[1].x, o3[2].x);
+          put(k2, o3[0].y, o3[1].y, o3[2].y);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < kN1; ++k) {
+          const int o = xown + kXk * k;
+          const float xv[3] = {ex0[o], ex1[o], x2[k]};
+          float o3[3] = {0.f, 0.f, 0.f};
+          if (live) gm.apply(la + lb * kN1 + k * kN1 * kN1, cx[k], cw[k], xv, o3);
+          put(k, o3[0], o3[1], o3[2]);
+        }
       }
     }
     st_code4<OP>(bufT, cm_off<ESZ>(tid, 0, F::kLboT, F::kSboT), tt);
@@ -560,11 +582,12 @@ constexpr int kCtasGen =
 // results): measured on GB300 3 to 15% faster for the trilinear kinds (TF32
 // trilinear N = 3 143 -> 162, N = 15 192 -> 209 GDOF/s, BF16 N = 5 139 -> 152),
 // but for the 16-bit formats at N1 = 16, where its registers spill under the
-// three-CTA bound (BF16 223 -> 214); the stored and parallelepiped kinds' short
-// nodes gain nothing (BF16 parallelepiped N = 4 185 -> 169).
+// three-CTA bound (BF16 223 -> 214), and for the partial kind at N1 = 3 (TF32 116
+// -> 111); the stored and parallelepiped kinds' short nodes gain nothing (BF16
+// parallelepiped N = 4 185 -> 169).
 template <int N1, int KIND, int OP>
 constexpr bool kPackedGen =
-    (KIND == AX_GEOM_TRILINEAR || KIND == AX_GEOM_TRILINEAR_PARTIAL) && !(N1 == 16 && OP != 0);
+    (KIND == AX_GEOM_TRILINEAR || (KIND == AX_GEOM_TRILINEAR_PARTIAL && N1 != 3)) && !(N1 == 16 && OP != 0);
 
 template <int N1, int KIND, int OP>
 __global__ void __launch_bounds__(GShape<N1, OP>::THREADS, kCtasGen<N1, KIND, OP>)
@@ -756,12 +779,13 @@ __global__ void __launch_bounds__(GShape<N1, OP>::THREADS, kCtasGen<N1, KIND, OP
     // 4. geometry along the t-fiber of (i, j) = (la, lb), element le; 5. r, s, t into the operand buffers
     if (row_in_use) {
       uint32_t tt[N1];  // the t values, coded in the operand format
-      const bool live = EPB == 1 || le < nel;
-      const int64_t e = live ? e0 + le : e0;  // rows beyond the last element: its results are not stored
+      constexpr bool kPk = kPackedGen<N1, KIND, OP>;
+      const bool live = (kPk && EPB == 1) || le < nel;
+      const int64_t e = !kPk || live ? e0 + le : e0;  // packed: rows beyond the last element, see the order-7 kernel
       fiber::Geometry<P, N1, KIND> gm;
       gm.template prologue<false>(sgeo + le * (GW > 0 ? GW : 1), cx, cw, la, lb,
-                                  KIND == AX_GEOM_STORED ? geo + e * 7 * N3 : nullptr,
-                                  KIND == AX_GEOM_TRILINEAR_PARTIAL ? lam + e * N3 : nullptr, nullptr);
+                                  (KIND == AX_GEOM_STORED && (kPk || live)) ? geo + e * 7 * N3 : nullptr,
+                                  (KIND == AX_GEOM_TRILINEAR_PARTIAL && (kPk || live)) ? lam + e * N3 : nullptr, nullptr);
       auto put = [&](int k, float r, float s, float t) {
         st_op<OP>(bufR, cm_off<ESZ>(lb + N1 * k + F * le, la, G::LBO_R, G::SBO_R), r);
         st_op<OP>(bufS, cm_off<ESZ>(la + N1 * k + F * le, lb, G::LBO_S, G::SBO_S), s);
@@ -774,7 +798,7 @@ __global__ void __launch_bounds__(GShape<N1, OP>::THREADS, kCtasGen<N1, KIND, OP
         if (live) gm.apply(la + lb * N1 + k * F, cx[k], cw[k], xv, o3);
         put(k, o3[0], o3[1], o3[2]);
       };
-      if constexpr (kPackedGen<N1, KIND, OP>) {
+      if constexpr (kPk) {
         const fiber::Geometry2<N1, KIND> g2(gm);
 #pragma unroll
         for (int k = 0; k < N1 / 2; ++k) {
