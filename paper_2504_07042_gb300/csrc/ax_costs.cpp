@@ -1,7 +1,10 @@
 // Design instruction counts of the fiber-per-thread AxLocal kernels
 // (ax_fiber.cuh), per node, on the binding arithmetic pipe (FP64 pipe for
 // native FP64, FP32 pipe for native FP32 and double-word).  Used by
-// ax_query for the time-based roofline of Sec. 3.4.
+// ax_query for the time-based roofline of Sec. 3.4.  The double-word costs are
+// a fixed yardstick, so that fractions of it stay comparable: the kernels have
+// since come to need 10 instead of 12 operations for a multiply-accumulate and
+// 13 instead of 15 for a*b + c (dw.cuh), and their fractions rose accordingly.
 #include "ax_internal.h"
 
 namespace ax {
