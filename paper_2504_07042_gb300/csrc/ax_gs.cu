@@ -274,8 +274,8 @@ __global__ void __launch_bounds__(kRedThreads, kRedBlocks / 152)
 // brought up to date by finish_x.  Bound by HBM and L2 traffic and, in
 // float64, by the FP64 pipe (5 to 6 operations per node at 2 per clock and
 // SM).  Measured on GB300 per iteration at order 7, 4096 elements, against the
-// four launches of the general one: double-word 104 against 115 us (operator
-// 78, gather_update 27), float32 33 against 48 us (20 and 13).
+// four launches of the general one: double-word 100 against 115 us (operator
+// 75, gather_update 27), float32 33 against 48 us (20 and 13).
 // ---------------------------------------------------------------------------
 // gather_update's blocks per SM and nodes per thread whose loads are in flight
 // together.  Double: two nodes in 40 registers, so that 48 warps per SM keep
