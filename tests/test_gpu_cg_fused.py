@@ -101,3 +101,18 @@ def test_stops_inside_a_block(ax, orc):
         assert st == ax.AX_OK and rr <= rtol
         true = np.linalg.norm(b - A(x.cpu().numpy())) / np.linalg.norm(b)
         assert abs(true - rr) <= 1e-10
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -200, 2.0 ** 150])
+@pytest.mark.parametrize("N", [7, 11])
+def test_far_from_unit_scale(ax, orc, N, scale):
+    # a direction outside float32's exponent range: every block is read again,
+    # scaled; CG is linear in b and powers of two are exact, so the iterates
+    # scale with it
+    V, gid, ng, mask, A, inv, b, _ = _problem(orc, (3, 2, 2), N)
+    ref = _cg(A, b, inv, np.zeros(ng), 9)
+    op = ax.Ax(torch.from_numpy(V).to(DEV), N, "trilinear", "f64dw")
+    op.gs_setup(torch.from_numpy(gid).to(DEV), ng, torch.from_numpy(mask).to(DEV))
+    x = torch.zeros(ng, dtype=torch.float64, device=DEV)
+    op.pcg_solve(torch.from_numpy(b * scale).to(DEV), x, rtol=0.0, maxit=9)
+    assert np.max(np.abs(x.cpu().numpy() / scale - ref)) <= 1e-9 * np.max(np.abs(ref))
