@@ -315,6 +315,9 @@ constexpr int kMinCtas =
     (kShapeClass<P> >= 0 && shape_min_ctas(kShapeClass<P>, N1, KIND)) ? shape_min_ctas(kShapeClass<P>, N1, KIND)
     : (P::kRoll && (N1 == 16 || (N1 == 12 && KIND == AX_GEOM_TRILINEAR)))  ? 2
                                                                            : 0;
+// the same registers for the tile of twice the elements where the bound is above four CTAs
+template <class P, int N1, int KIND, int EM>
+constexpr int kMinCtasEm = EM > 1 && kMinCtas<P, N1, KIND> > 4 ? kMinCtas<P, N1, KIND> / EM : kMinCtas<P, N1, KIND>;
 
 // Trilinear kinds: whether an element's first 2 N1 threads compute the axis
 // terms of the geometry (Geometry::axis_terms) for all its threads.  Measured
@@ -1191,7 +1194,7 @@ __device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIN
 // the grid is capped (autotuner)
 // ---------------------------------------------------------------------------
 template <class P, int N1, int KIND, int EM>
-__global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads, kMinCtas<P, N1, KIND>)
+__global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads, kMinCtasEm<P, N1, KIND, EM>)
     ax_fiber_kernel(int64_t E, const typename P::S *__restrict__ geo, const typename P::S *__restrict__ lam,
                     const typename P::IO *__restrict__ X, typename P::IO *__restrict__ Y) {
   using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
