@@ -2,6 +2,7 @@
 // dispatch to the kernel translation units, status and error strings.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -71,6 +72,7 @@ ax::AxArgs make_args(ax_ctx *c, const void *X, void *Y, void *stream) {
   a.E = c->c.E;
   a.N = c->c.N;
   a.kind = c->c.kind;
+  a.op = c->c.id;
   a.geo = c->c.geo;
   a.lam = c->c.lam;
   a.err = c->c.kerr;
@@ -171,6 +173,8 @@ ax_status ax_setup(ax_ctx **out, int64_t E, int N, const double *vertices, ax_ge
 
   ax_ctx *c = new (std::nothrow) ax_ctx;
   if (!c) return fail(nullptr, AX_ENOMEM, "ax_setup: host allocation failed");
+  static std::atomic<uint64_t> contexts{0};
+  c->c.id = ++contexts;
   c->c.E = E;
   c->c.N = N;
   c->c.N1 = (int)N1;

@@ -539,7 +539,7 @@ struct PcgWork {
   const void *graph_b = nullptr;  // the (b, x, preconditioner, operator, form) the graph was captured for
   void *graph_x = nullptr;
   bool graph_jac = false;
-  const void *graph_op = nullptr;
+  uint64_t graph_op = 0;  // AxArgs::op
   bool graph_fused = false;
   bool jac = false;  // Jacobi on: inv holds the inverted diagonal
   T *inv_or_null() const { return jac ? inv : nullptr; }
@@ -684,7 +684,7 @@ static cudaError_t pcg_core(const GsPlan &P, const AxArgs &base, cudaError_t (*l
     a.stream = cs;
     if (e == cudaSuccess && maxit >= kCheck &&
         (!W.exec || W.graph_b != (const void *)b || W.graph_x != (void *)x || W.graph_jac != W.jac ||
-         W.graph_op != base.geo || W.graph_fused != fused)) {
+         W.graph_op != base.op || W.graph_fused != fused)) {
       if (W.exec) cudaGraphExecDestroy(W.exec);
       W.exec = nullptr;
       cudaGraph_t graph = nullptr;
@@ -698,7 +698,7 @@ static cudaError_t pcg_core(const GsPlan &P, const AxArgs &base, cudaError_t (*l
         W.graph_b = b;
         W.graph_x = x;
         W.graph_jac = W.jac;
-        W.graph_op = base.geo;
+        W.graph_op = base.op;
         W.graph_fused = fused;
       }
     }

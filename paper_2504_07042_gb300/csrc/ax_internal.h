@@ -49,6 +49,7 @@ struct Ctx {
   ax_geom_kind kind = AX_GEOM_STORED;
   ax_precision prec = AX_FP64;
   int device = 0;
+  uint64_t id = 0;  // of this context, never given to another one in the process (AxArgs::op)
   // geometry record, in the storage type of the precision:
   //   STORED: factors [E][7][n3]; TRILINEAR(_PARTIAL): vertices [E][24];
   //   PARALLELEPIPED: constants [E][8]; PARTIAL additionally lam [E][n3].
@@ -99,6 +100,9 @@ struct AxArgs {
   int64_t E = 0;
   int N = 0;
   ax_geom_kind kind = AX_GEOM_STORED;
+  // The context that geo, lam and err belong to (Ctx::id): what a captured
+  // launch is kept by, since a later context's arrays can get the same addresses.
+  uint64_t op = 0;
   const void *geo = nullptr;
   const void *lam = nullptr;
   const void *X = nullptr;
