@@ -880,8 +880,14 @@ ax_status batch_pcg(ax_batch *b, const T *bvec, T *x, double rtol, int maxit, in
       if (W.hS[m * kS + 6] == 0.0) all_done = false;
   }
   if (e == cudaSuccess) {
-    if (one_launch) seg_finish_x<<<RB, kThreads, 0, s>>>(sg, W.S, (const float *)W.p, (const float *)W.w, (float *)W.x);
-    e = cudaMemcpyAsync(x, W.x, sizeof(T) * n, cudaMemcpyDeviceToDevice, s);
+    // (after a wait that ran out, a mesh can stand between the two halves of an
+    // iteration, where x and the update it is owed do not belong together: the
+    // caller keeps the initial guess)
+    if (pstatus == 0) {
+      if (one_launch)
+        seg_finish_x<<<RB, kThreads, 0, s>>>(sg, W.S, (const float *)W.p, (const float *)W.w, (float *)W.x);
+      e = cudaMemcpyAsync(x, W.x, sizeof(T) * n, cudaMemcpyDeviceToDevice, s);
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(W.hS, W.S, sizeof(double) * kS * B, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
