@@ -338,8 +338,9 @@ ax_status ax_local_host(ax_ctx *c, const void *X_host, void *Y_host, void *strea
   // (mapped memory): the kernel reads X and writes Y over the host link
   // itself, so both directions stay busy for the whole call and no staging
   // copies are made.  Measured on GB300 (order 7, 131072 elements): FP32
-  // 1.84 -> 1.60 ms per call, 0.98 of the link's two-way bound; the
-  // float64-IO kernels (double-word, FP64), which compute longer per byte
+  // 1.84 -> 1.60 ms per call, 0.98 of the link's two-way bound, with the kernel
+  // made for it (fiber::XLink; the one that runs on device memory takes 1.96);
+  // the float64-IO kernels (double-word, FP64), which compute longer per byte
   // with fewer resident warps, slowed down reading over the link (3.55 ->
   // 4.58 ms) and keep the chunked copy pipeline below, as does other host
   // memory.
@@ -353,7 +354,9 @@ ax_status ax_local_host(ax_ctx *c, const void *X_host, void *Y_host, void *strea
       const char *xd = (const char *)px.devicePointer;
       char *yd = (char *)py.devicePointer;
       if (xd < yd + bytes && yd < xd + bytes) return fail(c, AX_EINVAL, "ax_local_host: X and Y overlap");
-      e = run_ax(c, make_args(c, xd, yd, s));
+      ax::AxArgs a = make_args(c, xd, yd, s);
+      a.link = true;
+      e = run_ax(c, a);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) return cuda_fail(c, e, "ax_local_host");
       return AX_OK;

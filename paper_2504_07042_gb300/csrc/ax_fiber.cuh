@@ -737,13 +737,28 @@ struct GeoWords {
   static constexpr int value = (KIND == AX_GEOM_STORED) ? 0 : (KIND == AX_GEOM_PARALLELEPIPED ? kParWords : kVertexWords);
 };
 
-// Sources of X: in place (element e's values at X[e n3 + m]), or formed from
-// the assembled vectors of a CG iteration (XCg).
+// Sources of X: in place (element e's values at X[e n3 + m]), in place in host
+// memory (XLink), or formed from the assembled vectors of a CG iteration (XCg).
 template <typename IO>
 struct XDirect {
-  static constexpr bool kCg = false;
+  static constexpr bool kCg = false, kLink = false;
   const IO *__restrict__ p;
   __device__ __forceinline__ IO operator[](int64_t m) const { return p[m]; }
+};
+// X and Y in page-locked host memory, read and written over the host link
+// (ax_local_host, float32): consecutive words by consecutive threads, both ways
+// through shared memory.  The accesses that are best against HBM and shared
+// memory are not against the link, which moves a line's pieces one by one and
+// waits longer for each.  Measured on GB300 (3.2e7 nodes each way, us per call,
+// with the plain kernel / with this one; the link alone takes about 750): order 7
+// trilinear 950 / 789 (its warps touch four 32-byte pieces of four lines,
+// Layout::row_of), parallelepiped 1010 / 793, partial 1120 / 787; stored order 1
+// 980 / 760, order 3 853 / 777, order 5 1130 / 990; trilinear order 5 1110 / 778,
+// order 15 838 / 804.
+template <typename IO>
+struct XLink {
+  static constexpr bool kCg = false, kLink = true;
+  const IO *__restrict__ p;
 };
 // The search direction of a CG iteration, formed at each local copy while it
 // is loaded: p_new[g] = z[g] + beta p[g].  The thread that loads a node's
@@ -752,7 +767,7 @@ struct XDirect {
 // than p, so every copy sees the same p.  Y is stored by rank (CgArgs).
 template <typename IO>
 struct XCg {
-  static constexpr bool kCg = true;
+  static constexpr bool kCg = true, kLink = false;
   static constexpr int kBatch = 8;  // nodes whose loads are in flight together
   const gidx *__restrict__ own;
   const gidx *__restrict__ rank;
@@ -880,6 +895,11 @@ __device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIN
   const int64_t own = e * n3 + qa + N1 * jt;  // node (qa, jt, 0); k: + k F
   constexpr bool kRegX = !P::kRoll;  // native arithmetic: the fiber's x stays in registers for D_t x
   V xt[kRegX ? N1 : 1];
+  // value m of the block in shared memory
+  auto place = [](int m) {
+    const int row = m / N1;  // row (j, k) of element row / F
+    return row / F * ES + row / N1 % N1 * Sh::PK + row % N1 * Sh::P + m % N1;
+  };
   bool wide = false;  // this thread's fiber (or row) lies outside the direct range
   constexpr bool kRows = kRowLoads<P, N1> && !XS::kCg;
   if constexpr (kRows) {
@@ -897,6 +917,13 @@ __device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIN
         dst[i] = P::st(P::from_io_direct(v));
       }
       wide |= tiny || !row_direct(hmax);
+    }
+  } else if constexpr (XS::kLink) {
+    static_assert(kRegX && !IDLE, "the float32 kernels");
+#pragma unroll
+    for (int s = 0; s < N1; ++s) {
+      const int m = tid + s * Sh::threads;
+      if (m < nel * n3) xs[place(m)] = P::st(P::from_io(X.p[e0 * n3 + m]));
     }
   } else if (live) {
     using IO = typename P::IO;
@@ -960,6 +987,10 @@ __device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIN
     }
   } else {
     __syncthreads();
+  }
+  if constexpr (XS::kLink) {
+#pragma unroll
+    for (int k = 0; k < N1; ++k) xt[k] = live ? P::ld(x_e + ft + k * str_t) : P::lit(0.0);
   }
   if constexpr (AXS) {
     // threads q < 2 N1 of each element: the N1 r-axis and N1 s-axis terms,
@@ -1178,10 +1209,21 @@ __device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIN
         if constexpr (XS::kCg) {
           Y[at[k]] = y;
           xy += P::ld(x_e + sidx) * y;  // X still lies where it was loaded
+        } else if constexpr (XS::kLink) {
+          x_e[sidx] = P::st(y);  // x is no longer read
         } else {
           Y[own + k * F] = y;
         }
       }
+    }
+  }
+
+  if constexpr (XS::kLink) {
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < N1; ++s) {
+      const int m = tid + s * Sh::threads;
+      if (m < nel * n3) Y[e0 * n3 + m] = P::ld(xs + place(m));
     }
   }
 
@@ -1216,6 +1258,38 @@ __global__ void __launch_bounds__(Shape<N1, EM, kEpb<P, N1, KIND>>::threads, kMi
     const int64_t e0 = blk * EPB;
     const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
     fiber_block<P, N1, KIND, EM, false>(sm, tid, e0, nel, geo, lam, XDirect<typename P::IO>{X}, Y);
+  }
+}
+
+// Where ax_local_host runs this kernel on host memory: float32 (with float64
+// values the copies by chunks are faster), but for the recompute kinds of order
+// 2, whose blocks of 14 elements end in the middle of a line whatever the order
+// of the accesses (trilinear: the plain kernel 932 us, this one 968).
+template <class P, int N1, int KIND>
+constexpr bool kHasLink = sizeof(typename P::IO) == 4 && !(N1 == 3 && KIND != AX_GEOM_STORED);
+
+// The same with X and Y in host memory (XLink).
+template <class P, int N1, int KIND>
+__global__ void __launch_bounds__(Shape<N1, 1, kEpb<P, N1, KIND>>::threads, kMinCtas<P, N1, KIND>)
+    ax_fiber_link_kernel(int64_t E, const typename P::S *__restrict__ geo, const typename P::S *__restrict__ lam,
+                         const typename P::IO *__restrict__ X, typename P::IO *__restrict__ Y) {
+  using Sh = Shape<N1, 1, kEpb<P, N1, KIND>>;
+  using Buf = FiberSmem<P, N1, KIND, 1>;
+  using S = typename P::S;
+  constexpr int EPB = Sh::EPB;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ S sgeo[EPB][Buf::GWD];
+  __shared__ S sax[Buf::AXS ? EPB : 1][Buf::AXD];
+  Buf sm;
+  sm.xs = (S *)smem_raw;
+  sm.sgeo = &sgeo[0][0];
+  sm.sax = &sax[0][0];
+  sm.sexp = nullptr;
+  const int64_t nblk = (E + EPB - 1) / EPB;
+  for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    const int64_t e0 = blk * EPB;
+    const int nel = (int)((E - e0) < EPB ? (E - e0) : EPB);
+    fiber_block<P, N1, KIND, 1, false>(sm, threadIdx.x, e0, nel, geo, lam, XLink<typename P::IO>{X}, Y);
   }
 }
 
@@ -1349,24 +1423,29 @@ size_t launch_smem(const void *kernel) {
   return smem;
 }
 
-template <class P, int N1, int KIND, int EM>
+template <class P, int N1, int KIND, int EM, bool LINK = false>
 cudaError_t launch_ax_em(const AxArgs &a) {
   using Sh = Shape<N1, EM, kEpb<P, N1, KIND>>;
+  constexpr auto kernel = [] {
+    if constexpr (LINK)
+      return ax_fiber_link_kernel<P, N1, KIND>;
+    else
+      return ax_fiber_kernel<P, N1, KIND, EM>;
+  }();
   const int64_t nblk = (a.E + Sh::EPB - 1) / Sh::EPB;
   if (nblk <= 0) return cudaSuccess;
   const int64_t grid = a.grid > 0 && a.grid < nblk ? a.grid : nblk;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  static const size_t smem = launch_smem<P, N1, KIND, EM>((const void *)ax_fiber_kernel<P, N1, KIND, EM>);
+  static const size_t smem = launch_smem<P, N1, KIND, EM>((const void *)kernel);
   // per instantiation; static shared memory counts against the same 48 KB
   // default, so the attribute is set whatever the dynamic size
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(ax_fiber_kernel<P, N1, KIND, EM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  ax_fiber_kernel<P, N1, KIND, EM><<<(unsigned)grid, Sh::threads, smem, a.stream>>>(
+  kernel<<<(unsigned)grid, Sh::threads, smem, a.stream>>>(
       a.E, (const typename P::S *)a.geo, (const typename P::S *)a.lam, (const typename P::IO *)a.X,
       (typename P::IO *)a.Y);
   return cudaGetLastError();
@@ -1414,6 +1493,9 @@ cudaError_t launch_fiber_n(const AxArgs &a, double *G_out) {
       return launch_ax_cg<P, N1, KIND>(a);
     else
       return cudaErrorNotSupported;
+  }
+  if constexpr (kHasLink<P, N1, KIND>) {
+    if (a.link) return launch_ax_em<P, N1, KIND, 1, true>(a);
   }
   if constexpr (P::kTiles > 1) {
     if (a.tile == 1) return launch_ax_em<P, N1, KIND, 2>(a);

@@ -108,6 +108,7 @@ struct AxArgs {
   const void *X = nullptr;
   void *Y = nullptr;
   cudaStream_t stream = nullptr;
+  bool link = false;  // X and Y lie in host memory (the float32 launchers have a kernel for it)
   int tile = 0;      // tile variant (elements per CTA: 0 = base, 1 = twice; FP32 only)
   int64_t grid = 0;  // CTAs to launch (0 = one per block of elements; fewer = persistent loop)
   const CgArgs *cg = nullptr;  // FP32 and double-word launchers: the CG form (E = 0 only prepares the kernel)
