@@ -343,7 +343,7 @@ constexpr bool kShareAxis = (KIND == AX_GEOM_TRILINEAR || KIND == AX_GEOM_TRILIN
 // packed geometry (Geometry2), measured on GB300: order 7 trilinear 258 -> 221
 // us for 131072 elements, order 5 stored 421 -> 366 us for 309808, 1.02 to 1.47
 // times at every order and kind of 3.2e7 nodes but the stored kind at order 1
-// (0.98).
+// (equal).
 struct Pitches {
   int P, PK, ES, vec;  // row, plane and element pitch; words per row access
 };
@@ -1141,12 +1141,18 @@ __device__ __forceinline__ typename P::IO fiber_block(const FiberSmem<P, N1, KIN
       gm.template prologue<AXS>(sgeo_z, cx, cw, i, j, KIND == AX_GEOM_STORED ? geo + eg * 7 * n3 : nullptr,
                                 KIND == AX_GEOM_TRILINEAR_PARTIAL ? lam + eg * n3 : nullptr, sax_z);
       // (threads beyond the last element work on the block's first one's
-      // geometry: no branch per node, their results are not stored)
+      // geometry: no branch per node, their results are not stored; but for the
+      // stored kind at order 1, where the loads are scheduled better with one:
+      // 162 -> 164.5 GDOF/s on 3.2e7 nodes)
+      constexpr bool kNodeBranch = N1 == 2 && KIND == AX_GEOM_STORED;
       auto node = [&](int k) {
         const int sidx = ft + k * str_t;
         const V xv[3] = {P::ld(r_e + sidx), P::ld(s_e + sidx), tf[k]};
         V o3[3];
-        gm.apply(i + j * N1 + k * N1 * N1, P::cst(cx + k), P::cst(cw + k), xv, o3);
+        if (!kNodeBranch || live)
+          gm.apply(i + j * N1 + k * N1 * N1, P::cst(cx + k), P::cst(cw + k), xv, o3);
+        else
+          o3[0] = o3[1] = o3[2] = P::lit(0.0);
         r_e[sidx] = P::st(o3[0]);
         s_e[sidx] = P::st(o3[1]);
         tf[k] = o3[2];
