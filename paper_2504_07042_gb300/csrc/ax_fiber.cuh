@@ -315,9 +315,17 @@ constexpr int kMinCtas =
     (kShapeClass<P> >= 0 && shape_min_ctas(kShapeClass<P>, N1, KIND)) ? shape_min_ctas(kShapeClass<P>, N1, KIND)
     : (P::kRoll && (N1 == 16 || (N1 == 12 && KIND == AX_GEOM_TRILINEAR)))  ? 2
                                                                            : 0;
-// the same registers for the tile of twice the elements where the bound is above four CTAs
+// The tile of twice the elements (float32): half the CTAs where the base tile's
+// bound would make its 512 threads spill (N1 = 8 at eight CTAs; N1 = 16 at two, 800
+// bytes: stored 299 -> 117 us for 1.6e7 nodes, trilinear 202 -> 100), and two CTAs
+// at N1 = 14, where the recompute kinds would otherwise take 82 to 86 registers
+// and run one (trilinear 123 -> 86, partial 123 -> 92).  The stored kind at N1 =
+// 12 keeps its four (90 against 100 us at two), at 14 the 108 registers it takes.
 template <class P, int N1, int KIND, int EM>
-constexpr int kMinCtasEm = EM > 1 && kMinCtas<P, N1, KIND> > 4 ? kMinCtas<P, N1, KIND> / EM : kMinCtas<P, N1, KIND>;
+constexpr int kMinCtasEm = EM == 1                                ? kMinCtas<P, N1, KIND>
+                           : N1 == 8 || N1 == 16                  ? kMinCtas<P, N1, KIND> / EM
+                           : N1 == 14 && KIND != AX_GEOM_STORED   ? 2
+                                                                  : kMinCtas<P, N1, KIND>;
 
 // Trilinear kinds: whether an element's first 2 N1 threads compute the axis
 // terms of the geometry (Geometry::axis_terms) for all its threads.  Measured
