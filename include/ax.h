@@ -281,8 +281,8 @@ ax_status ax_batch_set_wait(ax_batch *b, int64_t budget_ns, int stuck_mesh);
  *   tiles (direction and update of x fused into their loads) and gather +
  *   update chunks, each waiting (bounded) for its mesh's previous phase;
  *   a wait past its budget stops the solve with AX_ETIMEOUT and leaves
- *   x_global as it was.  (A batch with a
- *   node that no element has runs one launch per order group and phase.)
+ *   x_global as it was.  (Nodes that no element has take a second, small
+ *   kernel.)
  *   graph = 0: reference path, each mesh solved in turn with its own
  *   launches (pcg_solve on its per-mesh context).
  *   iters, relres: host arrays [B].  AX_ENOTCONV if a mesh hit maxit.

@@ -171,6 +171,27 @@ __global__ void __launch_bounds__(kThreads)
   block_sum((double)bb, pbb + blockIdx.x);
 }
 
+// First half of a fused iteration at the nodes that no element has, which no
+// AxLocal tile loads: p_new = z + beta p, x += alpha p (fiber::XCg).  Node g lies
+// in the block k with blo[k] <= g < bhi[k].
+__global__ void seg_bare(Seg sg, int nblk, int64_t n, const gidx *__restrict__ bare, const double *__restrict__ S,
+                         const float *__restrict__ z, const float *__restrict__ p, float *__restrict__ pn,
+                         float *__restrict__ x) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= n) return;
+  const int64_t g = bare[q];
+  int lo = 0, hi = nblk;  // blo[lo] <= g < blo[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) / 2;
+    (sg.blo[mid] <= g ? lo : hi) = mid;
+  }
+  const double *s = S + sg.bmesh[lo] * kS;
+  if (s[6] != 0.0) return;
+  const float alpha = (float)s[10], beta = (float)s[11];
+  x[g] += alpha * p[g];
+  pn[g] = z[g] + beta * p[g];
+}
+
 // x += alpha p after a mesh's last iteration: the update that the fused
 // iteration still owes (p: the direction of odd or even iterations)
 __global__ void __launch_bounds__(kThreads)
@@ -820,9 +841,9 @@ ax_status batch_pcg(ax_batch *b, const T *bvec, T *x, double rtol, int maxit, in
     seg_start<<<(B + 127) / 128, 128, 0, s>>>(B, W.S, rtol);
     e = cudaGetLastError();
   }
-  // capture one iteration: one persistent launch (float32, N <= 9, every node
-  // with a local copy), once for each order of the two direction vectors, or
-  // the per-phase launches
+  // capture one iteration: one persistent launch (float32, N <= 9; with a small
+  // one before it for the nodes that no element has), once for each order of the
+  // two direction vectors, or the per-phase launches
   const bool one_launch = sizeof(T) == 4 && b->use_persist && e == cudaSuccess && gs_fused_view(P, s);
   if (W.one_launch != one_launch) W.drop_graphs();
   W.one_launch = one_launch;
@@ -857,6 +878,8 @@ ax_status batch_pcg(ax_batch *b, const T *bvec, T *x, double rtol, int maxit, in
     cudaGraph_t graph = nullptr;
     e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
+      if (one_launch && P.n_bare)
+        seg_bare<<<(unsigned)((P.n_bare + 255) / 256), 256, 0, s>>>(sg, RB, P.n_bare, P.bare, W.S, v.z, v.p, v.pn, v.x);
       const cudaError_t e2 = one_launch ? persist::launch_iteration(*b->ps, v, s) : batch_iteration<T>(b, W, W.x, s);
       e = cudaStreamEndCapture(s, &graph);
       if (e == cudaSuccess) e = e2;
@@ -962,7 +985,7 @@ ax_status ax_batch_info(const ax_batch *b, int *persistent, int *local_launches,
   if (local_launches) *local_launches = b->use_persist ? 1 : groups;
   // grouped iteration: scatter, one AxLocal per group, gather + dot, 3 segmented
   // sums, update, convergence test, direction
-  if (iteration_launches) *iteration_launches = b->use_persist && b->gs.complete ? 1 : groups + 7;
+  if (iteration_launches) *iteration_launches = b->use_persist ? (b->gs.n_bare ? 2 : 1) : groups + 7;
   return AX_OK;
 }
 

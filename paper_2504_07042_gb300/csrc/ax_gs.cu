@@ -443,6 +443,10 @@ cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int6
     plan.complete &= off[g + 1] != 0;
     off[g + 1] += off[g];
   }
+  std::vector<gidx> bare;
+  for (int64_t g = 0; !plan.complete && g < n_global; ++g)
+    if (off[g + 1] == off[g]) bare.push_back((gidx)g);
+  plan.n_bare = (int64_t)bare.size();
   std::vector<gidx> idx((size_t)n_local), gid32((size_t)n_local), fill(off.begin(), off.end() - 1);
   for (int64_t m = 0; m < n_local; ++m) {
     const int64_t g = gid[m];
@@ -460,6 +464,11 @@ cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int6
     e = cudaMemcpyAsync(plan.idx, idx.data(), sizeof(gidx) * n_local, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && n_local)
     e = cudaMemcpyAsync(plan.gid, gid32.data(), sizeof(gidx) * n_local, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && plan.n_bare) {
+    e = cudaMalloc(&plan.bare, sizeof(gidx) * plan.n_bare);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(plan.bare, bare.data(), sizeof(gidx) * plan.n_bare, cudaMemcpyHostToDevice, s);
+  }
   if (e == cudaSuccess && mask_dev) {
     e = cudaMalloc(&plan.mask, n_global > 0 ? n_global : 1);
     if (e == cudaSuccess) e = cudaMemcpyAsync(plan.mask, mask_dev, n_global, cudaMemcpyDeviceToDevice, s);
@@ -469,7 +478,7 @@ cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int6
 }
 
 bool gs_fused_view(const GsPlan &plan, cudaStream_t s) {
-  if (!plan.complete) return false;
+  if (plan.n_local == 0) return false;
   if (plan.own) return true;
   if (cudaMalloc(&plan.own, sizeof(gidx) * 2 * plan.n_local) != cudaSuccess) {
     cudaGetLastError();  // no room for it: the general iteration
@@ -487,6 +496,7 @@ void gs_free(GsPlan &plan) {
   cudaFree(plan.idx);
   cudaFree(plan.gid);
   cudaFree(plan.own);  // and rank
+  cudaFree(plan.bare);
   cudaFree(plan.mask);
   plan = GsPlan();
 }
@@ -594,7 +604,7 @@ static cudaError_t pcg_iteration(const GsPlan &P, const AxArgs &a, cudaError_t (
 // global node has a local copy to own it (a node without one is touched by
 // the general iteration's vector kernels only).
 static bool fused_ok(const GsPlan &P, cudaError_t (*launch)(const AxArgs &), cudaStream_t s) {
-  return (launch == launch_ax_fp32 || launch == launch_ax_dw) && gs_fused_view(P, s);
+  return (launch == launch_ax_fp32 || launch == launch_ax_dw) && P.complete && gs_fused_view(P, s);
 }
 
 // One fused CG iteration (two launches) on stream s; k: its number since the

@@ -35,6 +35,8 @@ struct GsPlan {
   gidx *idx = nullptr;  // [n_local], local indices grouped by global node, increasing within a group
   gidx *gid = nullptr;  // [n_local], global id of every local node
   bool complete = false;  // every global node has a local copy
+  gidx *bare = nullptr;   // [n_bare] the global nodes without one, increasing
+  int64_t n_bare = 0;
   // The fused CG iteration's view of the same map (gs_fused_view, built by the
   // first solve that runs it): own[m] = gid[m], sign bit set where m is the
   // first local copy of its node; rank[idx[q]] = q, the place of a local copy
@@ -159,8 +161,9 @@ cudaError_t setup_diag(const Ctx &c, const double *vertices, void *diag, bool f6
 // Gather-scatter and CG (ax_gs.cu).
 cudaError_t gs_build(GsPlan &plan, const int64_t *gid_dev, int64_t n_local, int64_t n_global, const uint8_t *mask_dev,
                      cudaStream_t s, int64_t *bad_ids);
-// Whether the fused CG iteration can run on the plan, building own and rank
-// on stream s if they are not there yet (false too when there is no room).
+// Whether own and rank of the plan are there, building them on stream s if not
+// (false when there is no room).  They say nothing of the nodes without a local
+// copy: a fused iteration updates those by itself or needs a complete plan.
 bool gs_fused_view(const GsPlan &plan, cudaStream_t s);
 void gs_free(GsPlan &plan);
 cudaError_t gs_assemble_run(const GsPlan &p, bool f64, void *Y, cudaStream_t s);
