@@ -24,10 +24,12 @@ namespace dw2 {
 
 using f2 = float2;
 
-// Each operation is written as PTX with an explicit .rn rounding modifier:
-// like the scalar __fadd_rn / __fmul_rn, such an instruction is never
-// contracted with a neighbour into a fused multiply-add, which would change
-// the rounding the error-free transformations rely on.
+// Each operation is written as PTX with an explicit .rn rounding modifier.
+// Unlike the scalar __fadd_rn / __fmul_rn, that alone does not keep a packed
+// product from being contracted with a sum that is its only use (see mac),
+// which would change the rounding the error-free transformations rely on: the
+// forms below are those that were measured to keep it, and
+// tests/test_gpu_dw.py compares their results with the scalar ones bit for bit.
 __device__ __forceinline__ f2 mul(f2 a, f2 b) {
   f2 r;
   asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n"
