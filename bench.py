@@ -222,6 +222,12 @@ def _pipe_peak(info, sm_mhz, sms=SM_COUNT):
     return FP32_LANES_PER_SM * sms * clk, "FP32 pipe"
 
 
+def _cost(op):
+    """ax_query's figures with the instructions that the kernel executes (the
+    design count would credit the pipe with work that it does not do)."""
+    return dict(op.ax_query(), pipe_ops_per_element=op.ax_executed_ops())
+
+
 def _roofline(info, ms, sm_mhz, hbm_gbs, sms=SM_COUNT):
     """Time-based roofline of Sec. 3.4: T_mem = bytes / measured HBM bandwidth,
     T_cmp = pipe instructions / pipe peak; frac = max(T_cmp, T_mem) / T_meas."""
@@ -413,7 +419,7 @@ def run(args):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
 
     op, X, Y, V = _build_case(ax, torch, dev, HEADLINE_N, HEADLINE_KIND, HEADLINE_PREC)
-    info = op.ax_query()
+    info = _cost(op)
     stream = torch.cuda.current_stream()
     E, n3 = op.E, op.n3
     fn = lambda: op.ax_local(X, Y, stream)  # noqa: E731
@@ -769,7 +775,7 @@ def run_sweep(ax, torch, dev, hbm, sm_mhz, sms=SM_COUNT):
                     if prec in ("tf32", "bf16", "fp16") and kind in ("stored", "partial"):
                         continue  # tensor-core contractions: the recompute kinds only
                     op, X, Y, _ = _build_case(ax, torch, dev, N, kind, prec, mesh)
-                    info = op.ax_query()
+                    info = _cost(op)
                     ms = _median_launch_ms(torch, lambda: op.ax_local(X, Y, stream), 20, 3, stream)
                     roof = _roofline(info, ms, sm_mhz, hbm, sms)
                     out.append({"N": N, "mesh": mesh, "kind": kind, "prec": prec, "E": op.E,

@@ -367,8 +367,8 @@ void ax_mlp_destroy(ax_mlp *m);
 
 /* Algorithmic cost of one ax_local call (per element): bytes moved to and
  * from HBM by the kernel's design, the paper's effective flops
- * F_ax = 12 N1^4 + 15 N1^3 (Table 2), and the arithmetic instructions the
- * kernel issues per element on its binding pipe (FP64 or FP32 lanes). */
+ * F_ax = 12 N1^4 + 15 N1^3 (Table 2), and the arithmetic instructions per
+ * element of the method's design on its binding pipe (FP64 or FP32 lanes). */
 typedef struct {
   int64_t E;
   int N;
@@ -380,6 +380,12 @@ typedef struct {
   int pipe;  /* 0 = FP64 pipe, 1 = FP32 pipe, 2 = tensor pipe */
 } ax_info;
 ax_status ax_query(const ax_ctx *c, ax_info *info);
+
+/* The instructions per element that the kernel executes on that pipe: what a
+ * rate or a fraction of the pipe's peak is formed with.  Below the design count
+ * for AX_F64DW, whose arithmetic has since become shorter (order 7 trilinear
+ * 793 per node instead of 890.5); the same for the other precisions. */
+ax_status ax_executed_ops(const ax_ctx *c, double *ops_per_element);
 
 /* Message for the last failed call on this context (or on context creation
  * when c is NULL).  Owned by the library; valid until the next call. */

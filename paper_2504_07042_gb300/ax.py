@@ -111,6 +111,8 @@ _lib.ax_mlp_destroy.argtypes = [_vp]
 _lib.ax_mlp_destroy.restype = None
 _lib.ax_query.argtypes = [_vp, ctypes.POINTER(ax_info)]
 _lib.ax_query.restype = _int
+_lib.ax_executed_ops.argtypes = [_vp, ctypes.POINTER(_dbl)]
+_lib.ax_executed_ops.restype = _int
 _lib.ax_last_error.argtypes = [_vp]
 _lib.ax_last_error.restype = ctypes.c_char_p
 _lib.ax_status_string.argtypes = [_int]
@@ -119,6 +121,7 @@ _lib.ax_destroy.argtypes = [_vp]
 _lib.ax_destroy.restype = None
 
 EXPORTS = ("ax_setup", "ax_local", "ax_local_host", "ax_local_host_static", "ax_factors", "ax_node_coords", "ax_query",
+           "ax_executed_ops",
            "gs_setup", "gs_assemble", "gs_gather", "gs_scatter", "ax_mass", "ax_diag", "pcg_solve", "pcg_solve_mixed",
            "ax_batch_setup", "ax_batch_sizes", "ax_batch_local", "ax_batch_tune", "ax_batch_pcg",
            "ax_batch_last_error", "ax_batch_destroy",
@@ -269,6 +272,12 @@ class Ax:
         info = ax_info()
         _check(_lib.ax_query(self.ctx, ctypes.byref(info)), self.ctx)
         return {k: getattr(info, k) for k, _ in ax_info._fields_}
+
+    def ax_executed_ops(self) -> float:
+        """Instructions per element that the kernel executes on its binding pipe."""
+        ops = _dbl(0.0)
+        _check(_lib.ax_executed_ops(self.ctx, ctypes.byref(ops)), self.ctx)
+        return ops.value
 
     def ax_destroy(self):
         if self.ctx:

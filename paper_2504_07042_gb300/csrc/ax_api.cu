@@ -470,6 +470,12 @@ ax_status ax_query(const ax_ctx *c, ax_info *info) {
   return AX_OK;
 }
 
+ax_status ax_executed_ops(const ax_ctx *c, double *ops_per_element) {
+  if (!c || !ops_per_element) return AX_EINVAL;
+  *ops_per_element = ax::executed_ops_per_node(c->c.N1, (int)c->c.kind, (int)c->c.prec) * (double)c->c.n3;
+  return AX_OK;
+}
+
 ax_status gs_setup(ax_ctx *c, const int64_t *global_id, int64_t n_global, const uint8_t *dirichlet_mask,
                    void *stream) {
   if (!c) return fail(nullptr, AX_EINVAL, "gs_setup: context is NULL");

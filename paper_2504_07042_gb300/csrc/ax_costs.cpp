@@ -1,24 +1,37 @@
 // Design instruction counts of the fiber-per-thread AxLocal kernels
 // (ax_fiber.cuh), per node, on the binding arithmetic pipe (FP64 pipe for
-// native FP64, FP32 pipe for native FP32 and double-word).  Used by
-// ax_query for the time-based roofline of Sec. 3.4.  The double-word costs are
-// a fixed yardstick, so that fractions of it stay comparable: the kernels have
-// since come to need 10 instead of 12 operations for a multiply-accumulate and
-// 13 instead of 15 for a*b + c (dw.cuh), and their fractions rose accordingly.
+// native FP64, FP32 pipe for native FP32 and double-word), for the time-based
+// roofline of Sec. 3.4.  Two counts:
+//   executed_ops_per_node  what the kernels execute, with the costs of the
+//                          present arithmetic (dw.cuh): the one to divide by a
+//                          time or a pipe rate.  Order 7 trilinear in
+//                          double-word: 793.0, against 800.1 by ncu's per-opcode
+//                          counts (FADD 390.9, FFMA 145.5, FMUL 53.8, and FFMA2
+//                          63, FADD2 36, FMUL2 6 doing two each).
+//   pipe_ops_per_node      the design count of the textbook sequences (12
+//                          operations for a multiply-accumulate, 15 for a*b + c,
+//                          14 for a quotient), which ax_query reports: a fixed
+//                          measure of an operator's arithmetic, not of what a
+//                          pipe was busy with.
 #include "ax_internal.h"
 
 namespace ax {
 
-double pipe_ops_per_node(int N1, int kind, int prec) {
+namespace {
+// double-word multiply-accumulate, a*b + c and quotient
+struct Costs {
+  double mac, fma, div;
+};
+double count(int N1, int kind, int prec, const Costs &k) {
   const bool dwp = (prec == AX_F64DW);
   const bool tc = (prec == AX_TF32 || prec == AX_BF16 || prec == AX_FP16);
   // cost of one scalar op in the arithmetic (dw.cuh): normalised sum, sum
   // without the final Fast2Sum, product, first product of an accumulator,
   // multiply-accumulate, finalisation, a*b + c, sum of two accumulators
   const double add = dwp ? 11.0 : 1.0, lazy = dwp ? 8.0 : 1.0, mul = dwp ? 9.0 : 1.0;
-  const double mul0 = dwp ? 4.0 : 1.0, mac = dwp ? 12.0 : 1.0, fin = dwp ? 3.0 : 0.0;
-  const double fma = dwp ? 15.0 : 1.0, accsum = dwp ? 8.0 : 1.0;
-  const double div = dwp ? 14.0 : 8.0;
+  const double mul0 = dwp ? 4.0 : 1.0, mac = dwp ? k.mac : 1.0, fin = dwp ? 3.0 : 0.0;
+  const double fma = dwp ? k.fma : 1.0, accsum = dwp ? 8.0 : 1.0;
+  const double div = dwp ? k.div : 8.0;
   // one even-odd fiber product of length N1 (c = N1/2 output pairs): 2c
   // even/odd sums, N1 accumulators started by a product, the remaining
   // terms as multiply-accumulates, each output pair formed from its two
@@ -67,5 +80,9 @@ double pipe_ops_per_node(int N1, int kind, int prec) {
   }
   return ops;
 }
+}  // namespace
+
+double pipe_ops_per_node(int N1, int kind, int prec) { return count(N1, kind, prec, {12.0, 15.0, 14.0}); }
+double executed_ops_per_node(int N1, int kind, int prec) { return count(N1, kind, prec, {10.0, 13.0, 12.0}); }
 
 }  // namespace ax

@@ -144,8 +144,10 @@ cudaError_t upload_tables_fp32(int device);
 cudaError_t upload_tables_dw(int device);
 cudaError_t upload_tables_setup(int device);
 
-// Binding-pipe instructions per node of the AxLocal kernel (design count).
+// Binding-pipe instructions per node of the AxLocal kernel: the design count,
+// and what the kernel executes (ax_costs.cpp).
 double pipe_ops_per_node(int N1, int kind, int prec);
+double executed_ops_per_node(int N1, int kind, int prec);
 
 // Setup kernels (FP64, ax_setup.cu).  flags: device int[4] zeroed by the caller:
 //   [0] count of GLL nodes with det J <= 0, [1] count of non-affine elements,
