@@ -706,12 +706,13 @@ ax_status ax_batch_tune(ax_batch *b, int *tiles, int64_t *grids, void *stream) {
 
 namespace {
 
-// Work of the batched solve, kept between calls: vectors (its own x, so that
+// Work of the batched solve, kept from the first call until the batch goes: vectors (its own x, so that
 // the captured iterations refer to nothing of the caller's), scalars, graphs,
 // and, as pcg_solve keeps it in its context, the inverted Jacobi diagonal, a
 // function of the meshes alone.  Allocating and freeing it, capturing, and the
 // diagonal's FP64 arithmetic took 2.6 of a call's 6.6 ms (16 meshes, 7.7e6
-// local nodes, 20 iterations).
+// local nodes, 20 iterations); the first call still pays for them (6.1 ms, the
+// later ones 4.0).
 template <typename T>
 struct BWork {
   T *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *w = nullptr, *Ul = nullptr, *Yl = nullptr, *inv = nullptr;

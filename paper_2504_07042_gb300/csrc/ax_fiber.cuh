@@ -349,7 +349,7 @@ constexpr bool kShareAxis = (KIND == AX_GEOM_TRILINEAR || KIND == AX_GEOM_TRILIN
 // padded rows alone need 22 at N1 = 4, 8 and 16, 23 to 28 at 6, 9, 10 and 12
 // to 14, 34 to 77 at 5, 7, 11 and 15.  Together with the loads below and the
 // packed geometry (Geometry2), measured on GB300: order 7 trilinear 258 -> 221
-// us for 131072 elements, order 5 stored 421 -> 366 us for 309808, 1.02 to 1.47
+// us for 131072 elements, order 5 stored 434 -> 366 us for 309808, 1.02 to 1.47
 // times at every order and kind of 3.2e7 nodes but the stored kind at order 1
 // (equal).
 struct Pitches {

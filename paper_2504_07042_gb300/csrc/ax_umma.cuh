@@ -230,7 +230,8 @@ __device__ __forceinline__ void st_op(unsigned char *base, uint32_t off, float v
 
 // The geometry at two nodes per instruction stream (fiber::Geometry2, the same
 // results): measured on GB300 at order 7 11 to 16% faster for the trilinear kind
-// (TF32 196 -> 217 GDOF/s), 21 to 29% for the partial, 2 to 11% for the
+// (TF32 196 -> 217 GDOF/s), 21 to 29% for the partial (TF32 157 -> 191, BF16 161 ->
+// 202, the 40 to 56 bytes of stack that it takes there included), 2 to 11% for the
 // parallelepiped and 6 to 8% for the stored kind with 16-bit operands, but 3%
 // slower for the stored kind in TF32 (182 -> 176).
 template <int KIND, int OP>
@@ -584,7 +585,10 @@ constexpr int kCtasGen =
 // but for the 16-bit formats at N1 = 16, where its registers spill under the
 // three-CTA bound (BF16 223 -> 214), and for the partial kind at N1 = 3 (TF32 116
 // -> 111); the stored and parallelepiped kinds' short nodes gain nothing (BF16
-// parallelepiped N = 4 185 -> 169).
+// parallelepiped N = 4 185 -> 169).  At N1 = 14 and 15 the packed form spills as
+// well, up to 104 bytes, and is the faster one all the same: N = 13 trilinear TF32
+// 148 -> 151, BF16 163 -> 168; N = 14 164 -> 172 and 177 -> 184, partial 143 -> 149
+// and 149 -> 158.
 template <int N1, int KIND, int OP>
 constexpr bool kPackedGen =
     (KIND == AX_GEOM_TRILINEAR || (KIND == AX_GEOM_TRILINEAR_PARTIAL && N1 != 3)) && !(N1 == 16 && OP != 0);
