@@ -307,12 +307,15 @@ constexpr int kEpb =
 // per SM, 5-30% slower); the double-word trilinear kernel at N1 = 12
 // (288-thread CTAs) likewise to two CTAs (96 registers and some spills
 // instead of 119 registers and one CTA: 33% faster; the partial kind
-// measured 5% slower so and keeps its allocation); the exceptions of
+// measured 5% slower so and keeps its allocation); native FP64's partial kind at
+// N1 = 7 to two CTAs of 392 threads (72 registers; unbounded it takes 102 and runs
+// one: 1181 -> 1149 us for 8.4e6 nodes, 197 -> 194.6 for 1e6); the exceptions of
 // shape_min_ctas.  Elsewhere no bound is given: even an explicit 1 changes
 // the register allocation for the worse.
 template <class P, int N1, int KIND>
 constexpr int kMinCtas =
     (kShapeClass<P> >= 0 && shape_min_ctas(kShapeClass<P>, N1, KIND)) ? shape_min_ctas(kShapeClass<P>, N1, KIND)
+    : (!P::kRoll && sizeof(typename P::S) == 8 && N1 == 7 && KIND == AX_GEOM_TRILINEAR_PARTIAL)            ? 2
     : (P::kRoll && (N1 == 16 || (N1 == 12 && KIND == AX_GEOM_TRILINEAR)))  ? 2
                                                                            : 0;
 // The tile of twice the elements (float32): half the CTAs where the base tile's
